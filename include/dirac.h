@@ -192,7 +192,9 @@ dirac_status dirac_apply_assembled(dirac_op* op, int sign, const void* x_dev, vo
  * FP32 copies of S and H0 per kappa, FP32 coupling values (precision 1: the FP32 rounding of the
  * FP64 assembly; precision 2: the hi words of the double-float assembly), and the kernel the
  * solve uses: the owner/gather passes for order-7 splines, the factorised apply when
- * dirac_op_set_factorised is on, else the per-row kernel.  Assembles the coupling values for t
+ * dirac_op_set_factorised is on, else the per-row kernel; on large precision-2 systems (order 7;
+ * from about 150 channels at N = 1000 or 400 at N = 250 on, all mu) the factorised product with the angular sums first, which steps
+ * at tolerances below 1e-11 use, too, while those above keep the forms named before.  Assembles the coupling values for t
  * first.  x_dev, y_dev: device complex64[n] (interleaved re, im floats, library order), must not
  * alias.  Synchronises the op's stream (it reads the error word of the bounded bulk-copy waits).
  * Errors: DIRAC_E_ARG (NULL, aliasing, sign not +-1, precision 0), DIRAC_E_CUDA. */
@@ -205,7 +207,9 @@ dirac_status dirac_precond_apply32(dirac_op* op, const void* r_dev, void* z_dev)
 
 /* The refinement residual of a step, r = A_-(t) psi - A_+(t) x (Eq. solPsi), computed as the step
  * computes it: precision 2 in double-float by the owner/gather passes (order-7 splines) or the
- * per-row residual kernel, precision 0 and 1 in FP64 (b = A_- psi, then r = b - A_+ x).
+ * per-row residual kernel, precision 0 and 1 in FP64 (b = A_- psi, then r = b - A_+ x).  On large
+ * precision-2 systems (see dirac_apply32) the product has the angular sums first; a step at a
+ * tolerance of 1e-11 or above still takes the owner/gather passes, whose rounding error is the larger.
  * Assembles the coupling values for t first.  psi_dev, x_dev, r_dev: device complex128[n]; r_dev
  * must alias neither.  bnorm (host, nullable) receives ||A_- psi||_2 as the step's tolerance test
  * uses it (precision 2: from FP32 products).  Synchronises the op's stream.  Errors: DIRAC_E_ARG,
@@ -346,7 +350,8 @@ int dirac_op_get_schedule(const dirac_op* op, int complex64);   /* -1 for a NULL
  * production size), 2 the per-channel form.  The first switch to a form builds its tables on the
  * host and allocates the products of two radial tiles (2 x channels x multipoles x 4 x 64 x 2
  * complex64) and, for form 1, the FP32 hi words of the radial bands (written by every later
- * assembly) and the subgroup item tables.  DIRAC_E_ARG for other precisions, spline orders or
+ * assembly) and the subgroup item tables.  Where a product has the angular sums first (large systems,
+ * see dirac_apply32) modes 0 and 1 take it alike.  DIRAC_E_ARG for other precisions, spline orders or
  * modes; DIRAC_E_CUDA if the subgroup form's shared-memory need exceeds the device's limit.  The
  * input and output vectors of an apply must not alias. */
 dirac_status dirac_op_set_factorised(dirac_op* op, int enable);

@@ -128,6 +128,7 @@ void collect_phases(dirac_op* op)
 // ---- launch helpers ------------------------------------------------------------------------
 int apply_parts(const dirac_op* op, const Krylov& K)
 {
+    if (op->use_ang && (K.prec == 0 || op->fact32 != 2)) return rad_parts(K.prec, op->ov.n1, op->nrad_lanes);
     if (K.prec == 1 && op->fact32 == 1) return grid_for(op->ov.n1, FTR) * op->nfsub;
     if (K.prec == 1 && op->fact32 == 2) return grid_for(op->ov.n1, FTR) * op->ov.nch;
     return (K.prec == 1 && op->part_own) ? op->nparts_own : op->nparts_apply;
@@ -138,10 +139,18 @@ void k_apply_launch(dirac_op* op, const Krylov& K, int sign, const void* x, void
 {
     PhaseScope ps(op, K.prec == 0 ? DIRAC_PHASE_APPLY : DIRAC_PHASE_APPLY32, 1);
     dim3 grid(op->ov.nch, grid_for(op->ov.n1, 128));
-    if (K.prec == 0)
+    if (K.prec == 0 && op->use_ang) {
+        op->launches++;
+        launch_ang64(op->st, op->ov, op->ang4, op->ang_c64, op->rad_lanes, op->nrad_lanes, op->Ed, (const double*)K.S,
+                     (const double*)K.H, sign, x, op->ang_S, y, bsub, dv, pdot, pnrm, skip);
+    } else if (K.prec == 0)
         launch_apply_t<double>(grid, op->st, op->ov, (const double*)K.S, (const double*)K.H, sign, x,
                                (const double*)K.W, y, bsub, dv, pdot, pnrm, skip);
-    else if (op->fact32 == 1)
+    else if (op->use_ang && op->fact32 != 2) {
+        op->launches++;
+        launch_ang32(op->st, op->ov, op->ang4, op->ang_c32, op->rad_lanes, op->nrad_lanes, op->aset[op->acur].Ef,
+                     (const float*)K.S, (const float*)K.H, sign, x, op->ang_S, y, bsub, dv, pdot, pnrm, skip, nullptr);
+    } else if (op->fact32 == 1)
         launch_fact32_sub(op->st, op->ov, op->rad_lanes, op->nrad_lanes, op->fsub, op->nfsub, op->fsub_max,
                           op->fitem_off, op->fitem_coef, op->Ghi, op->pv.L, op->S32T, op->H32T, sign, x, op->Zf, y, bsub, dv,
                           pdot, pnrm, skip);
@@ -156,15 +165,20 @@ void k_apply_launch(dirac_op* op, const Krylov& K, int sign, const void* x, void
                               (const float*)K.W, y, bsub, dv, pdot, pnrm, skip);
 }
 
-// precision 2: pulse factors, combined bands and double-float coupling values of one buffer set,
-// on stream st (the op's stream, or the overlap stream)
+// precision 2: pulse factors and, of one buffer set, what the products in use read at this time: the
+// band entries of the factorised products, or the double-float coupling values; on stream st (the
+// op's stream, or the overlap stream)
 void launch_assemble_set(dirac_op* op, cudaStream_t st, const AsmSet& a)
 {
-    PhaseScope ps(op, DIRAC_PHASE_ASSEMBLE, op->npairs ? 4 : 2, st);
+    PhaseScope ps(op, DIRAC_PHASE_ASSEMBLE, op->use_ang ? 3 + (op->fact32 == 2) : op->npairs ? 4 : 2, st);
     k_time_factors<<<1, 128, 0, st>>>(op->pv, a.t_eval, a.s);
+    if (op->use_ang) {
+        launch_rad_entries(st, op->pv, op->ov.n1, a.s, a.Ef, a.Ex, nullptr, a.Ers);
+        if (op->fact32 != 2) return;   // the per-channel form reads the G bands
+    }
     int be = op->ov.n1 * op->ov.bd * 4;
     k_field_combine_df<<<dim3(grid_for(be, 256), op->pv.L * 4), 256, 0, st>>>(op->pv, be, a.s, a.Gdf, a.Ghi);
-    if (op->npairs) {
+    if (op->npairs && !op->use_ang) {
         if (op->asm_chunks) {
             launch_assemble_grp_df(st, op->ov, op->asm_chunks, op->asm_nchunks, op->asm_gpair, op->asm_gcoef,
                                    a.Gdf, a.Wh, a.Wl);
@@ -184,8 +198,12 @@ void launch_assemble(dirac_op* op)
         launch_assemble_set(op, op->st, op->aset[op->acur]);
         return;
     }
-    PhaseScope ps(op, DIRAC_PHASE_ASSEMBLE, op->npairs ? 4 : 2);
+    PhaseScope ps(op, DIRAC_PHASE_ASSEMBLE, op->use_ang ? 2 : op->npairs ? 4 : 2);
     k_time_factors<<<1, 128, 0, op->st>>>(op->pv, op->t_eval, op->s);
+    if (op->use_ang) {
+        launch_rad_entries(op->st, op->pv, op->ov.n1, op->s, nullptr, nullptr, op->Ed, nullptr);
+        return;
+    }
     int be = op->ov.n1 * op->ov.bd * 4;
     k_field_combine<<<dim3(grid_for(be, 256), op->pv.L * 4), 256, 0, op->st>>>(op->pv, be, op->s, op->G);
     if (op->npairs) {
@@ -197,12 +215,23 @@ void launch_assemble(dirac_op* op)
     }
 }
 
+static bool residual_offsets(const dirac_op* op);
+
 // y = A_sign x accurate to double precision (x, y, bsub complex128): native FP64 kernels, or the
 // double-float kernels in precision 2
 void apply_accurate(dirac_op* op, int sign, const void* x, void* y, const void* bsub, double* pnrm)
 {
     if (op->opts.precision != 2) {
         k_apply_launch(op, op->k64, sign, x, y, bsub, nullptr, nullptr, pnrm, nullptr);
+        return;
+    }
+    if (op->use_ang && !bsub) {
+        PhaseScope ps(op, DIRAC_PHASE_APPLY, 3);
+        const AsmSet& a = op->aset[op->acur];
+        launch_split_rows(op->st, op->ov.nch, op->ov.n1, (const double2*)x, nullptr, op->xsplit, nullptr, nullptr,
+                          op->ang_umax);
+        launch_ang_df(op->st, op->ov, op->angx, false, op->ang_cx, op->rad_lanes, op->nrad_lanes, a.Ex, a.Ers, op->Sdf,
+                      op->Htdf, sign, op->xsplit, op->ang_umax, op->xsplit, op->ang_S, (double2*)y, pnrm);
         return;
     }
     PhaseScope ps(op, DIRAC_PHASE_APPLY, 2);
@@ -217,7 +246,7 @@ void apply_accurate(dirac_op* op, int sign, const void* x, void* y, const void* 
 void rhs_accurate(dirac_op* op, const void* psi)
 {
     if (op->opts.precision == 2) {
-        if (op->part_rdf) {
+        if (op->need_b) {
             k_set_int<<<1, 1, 0, op->st>>>(op->need_b, 1);
             op->launches++;
         }
@@ -225,13 +254,13 @@ void rhs_accurate(dirac_op* op, const void* psi)
     }
     Krylov& K = op->k64;
     apply_accurate(op, -1, psi, K.b, nullptr, op->part_n);
-    finish(op, K.ks, 0, op->nparts_apply, nullptr, op->part_n, op->opts.max_iter);
+    finish(op, K.ks, 0, apply_parts(op, K), nullptr, op->part_n, op->opts.max_iter);
 }
 
-// the owner pass's accumulators: fixed-binade form (offsets) or Dot2 (dirac_op_set_residual_mode)
+// the residual's accumulators: fixed-binade form (offsets) or Dot2 (dirac_op_set_residual_mode)
 static bool residual_offsets(const dirac_op* op)
 {
-    if (!op->own_sig) return false;
+    if (!op->own_sig && !op->use_ang) return false;
     return op->resid_mode == 2 || (op->resid_mode == 0 && op->opts.tol >= 1e-11);
 }
 
@@ -243,7 +272,32 @@ void residual_accurate(dirac_op* op, const void* psi)
     Krylov& K = op->k64;
     if (op->opts.precision != 2) {
         apply_accurate(op, +1, K.x, K.r, K.b, op->part_n);
-        finish(op, K.ks, 1, op->nparts_apply, nullptr, op->part_n, op->opts.max_iter);
+        finish(op, K.ks, 1, apply_parts(op, K), nullptr, op->part_n, op->opts.max_iter);
+        return;
+    }
+    if (op->use_ang) {
+        // factorised form: no coupling values; b = A_- psi by the complex64 product on a step's first pass
+        const AsmSet& a = op->aset[op->acur];
+        const int np = rad_parts(2, op->ov.n1, op->nrad_lanes), np32 = rad_parts(1, op->ov.n1, op->nrad_lanes);
+        {
+            PhaseScope ps(op, DIRAC_PHASE_APPLY, 5);
+            launch_split_rows(op->st, op->ov.nch, op->ov.n1, (const double2*)psi, (const double2*)K.x, op->xsplit,
+                              op->vsplit, op->psi32, op->ang_umax);
+            {
+                PhaseScope po(op, DIRAC_PHASE_OWNER, 0);   // the double-float product alone
+                launch_ang_df(op->st, op->ov, op->angx, residual_offsets(op), op->ang_cx, op->rad_lanes, op->nrad_lanes,
+                              a.Ex, a.Ers, op->Sdf, op->Htdf, -1, op->xsplit, op->ang_umax, op->vsplit, op->ang_S,
+                              (double2*)K.r, op->part_n);
+            }
+            launch_ang32(op->st, op->ov, op->ang4, op->ang_c32, op->rad_lanes, op->nrad_lanes, a.Ef,
+                         (const float*)op->k32.S, (const float*)op->k32.H, -1, op->psi32, op->ang_S, op->b32, nullptr,
+                         nullptr, nullptr, op->part_n2, nullptr, op->need_b);
+        }
+        {
+            PhaseScope ps(op, DIRAC_PHASE_VECTOR, 1);
+            k_bnorm_if<<<1, 1024, 0, op->st>>>(K.ks, op->need_b, np32, op->part_n2);
+        }
+        finish(op, K.ks, 1, np, nullptr, op->part_n, op->opts.max_iter);
         return;
     }
     if (op->part_rdf) {
@@ -642,6 +696,199 @@ static dirac_status alloc_krylov(dirac_op* op, Krylov& K, int prec, double tol)
     return DIRAC_OK;
 }
 
+// Whether the products of this system have the factorised form.  The stored form's cost is its coupling
+// values, npairs n1; the factorised one's the radial pass, whose blocks (one per 32 channels and 32
+// slots) run the 6 L + 4 stages one after the other and fill the chip from about 304 blocks (two per SM)
+// on.  The ratio q of the two orders the systems by their gain.  Measured over |kappa| <= 2 .. 30, N = 40
+// .. 1000, l <= 1 .. 6, all mu and |mu| = 1/2, a call that assembles its time (stored time / factorised
+// time): from q = 40e3 on the residual gains 1.32 (|kappa| <= 10, N = 600, l <= 1) to 2.77 (production,
+// q = 143e3) and the complex64 apply 3.2 to 9; at 15e3 .. 25e3 the residual ranges over 0.90 .. 1.27.  In
+// FP64 the apply alone, of which a step has ten for one assembly, ranges over 0.94 (|kappa| <= 20, N = 250,
+// l <= 6) .. 1.66 above q = 85e3 and is the slower one below (0.59 .. 0.96 at 60e3 .. 84e3).  Few channels
+// per kappa (|mu| = 1/2) leave the lanes idle: q stays below 11e3 there.
+static bool ang_pays(const dirac_op* op)
+{
+    const int n1 = op->B.n1;   // (the view is not set yet)
+    const double blocks = (double)op->nrad_lanes * grid_for(n1, 32);
+    const double q = (double)op->npairs * n1 / ((6.0 * op->pv.L + 4.0) * std::max(1.0, blocks / 304.0));
+    if (op->opts.precision == 2) return q >= 40e3;
+    return op->opts.precision == 0 && q >= 85e3;
+}
+
+// Whether a step takes it, too.  A mixed step at tolerances of 1e-11 and above runs its residual on
+// offsets, and the error of the stored form's (up to 1.6e-12 ||b|| near a pulse's start, 1e-10 of psi once
+// solved for) is part of its states: it keeps the stored form and with it its results.  Below, on Dot2
+// sums, the states of the two forms agree to 5e-13.
+static bool ang_steps(const dirac_op* op)
+{
+    return op->ang && (op->opts.precision != 2 || op->opts.tol < 1e-11);
+}
+
+// Tables and buffers of the factorised products (kernels_ang.cu): kappa chunks of up to FLANE channels
+// for the radial pass, two per warp where they fit; for the angular pass lists of neighbouring channels
+// of one mu and one parity of the orbital l with, per multipole, the union of their partners and each
+// output's coefficients
+//   alpha = c tau A1(a, b) (of K_l(ka, kb)), beta = -c tau A2(a, b) (of KT_l(kb, ka)).
+// ord: the channels sorted by kappa slot.
+static dirac_status ang_setup(dirac_op* op, const std::vector<int>& ord, const std::vector<int>& kslot)
+{
+    const Basis& B = op->B;
+    const int nch = B.nch, L = op->pv.L, n1 = B.n1;
+    const double ct = B.p.c * 0.5 * op->opts.dt;
+    std::vector<RadChunk> ch1;
+    for (int i = 0; i < nch;) {
+        int j = i;
+        while (j < nch && kslot[ord[j]] == kslot[ord[i]] && j - i < FLANE) j++;
+        ch1.push_back(RadChunk{kslot[ord[i]], B.kap[ord[i]], i, j - i});
+        i = j;
+    }
+    // two chunks per block where their channels fit the lanes together: largest first, each paired
+    // with the largest unpaired chunk that still fits
+    std::stable_sort(ch1.begin(), ch1.end(), [](const RadChunk& p, const RadChunk& q) { return p.count > q.count; });
+    std::vector<char> used(ch1.size(), 0);
+    std::vector<RadPack> rl;
+    for (size_t i = 0; i < ch1.size(); i++) {
+        if (used[i]) continue;
+        used[i] = 1;
+        RadPack pk{};
+        pk.c[0] = ch1[i];
+        pk.c[1] = RadChunk{ch1[i].ks, ch1[i].kappa, ch1[i].first, 0};
+        for (size_t j = i + 1; j < ch1.size(); j++)
+            if (!used[j] && ch1[i].count + ch1[j].count <= FLANE) {
+                used[j] = 1;
+                pk.c[1] = ch1[j];
+                break;
+            }
+        rl.push_back(pk);
+    }
+    dirac_status e = upload(op, &op->rad_lanes, rl);
+    if (e) return e;
+    op->nrad_lanes = (int)rl.size();
+    if (!ang_pays(op)) return DIRAC_OK;
+    // per (channel, multipole): (partner, alpha, beta), partners ascending within each half of the list
+    struct Use { int b; double al, be; };
+    std::vector<std::vector<Use>> uses((size_t)nch * L);
+    for (size_t p = 0; p < B.pa.size(); p++) {
+        const int a = B.pa[p], b = B.pb[p];
+        for (int q = B.pterm_start[p]; q < B.pterm_start[p + 1]; q++) {
+            const PairTerm& t = B.pterm[q];
+            uses[(size_t)a * L + t.l].push_back(Use{b, ct * t.A1, -ct * t.A2});
+            uses[(size_t)b * L + t.l].push_back(Use{a, ct * t.A2, -ct * t.A1});
+        }
+    }
+    // channels ordered by mu, parity of the orbital l and |kappa|
+    auto parity = [&](int a) { return (B.kap[a] > 0 ? B.kap[a] : -B.kap[a] - 1) & 1; };
+    std::vector<int> chs(nch);
+    for (int a = 0; a < nch; a++) chs[a] = a;
+    std::stable_sort(chs.begin(), chs.end(), [&](int p, int q) {
+        if (B.tmu[p] != B.tmu[q]) return B.tmu[p] < B.tmu[q];
+        if (parity(p) != parity(q)) return parity(p) < parity(q);
+        if (std::abs(B.kap[p]) != std::abs(B.kap[q])) return std::abs(B.kap[p]) < std::abs(B.kap[q]);
+        return B.kap[p] < B.kap[q];
+    });
+    // lists of up to no neighbouring channels of one mu and parity; coefficients [item][no][4]
+    auto lists = [&](int no, AngList& v, std::vector<double>& coef) -> dirac_status {
+        std::vector<std::vector<int>> groups;
+        for (int i = 0; i < nch;) {
+            std::vector<int> g;
+            while ((int)g.size() < no && i < nch &&
+                   (g.empty() || (B.tmu[chs[i]] == B.tmu[g[0]] && parity(chs[i]) == parity(g[0]))))
+                g.push_back(chs[i++]);
+            g.resize(no, -1);
+            groups.push_back(g);
+        }
+        // the heaviest lists first, so that the long blocks start in the first wave
+        auto weight = [&](const std::vector<int>& g) {
+            size_t w = 0;
+            for (int a : g)
+                for (int l = 0; a >= 0 && l < L; l++) w += uses[(size_t)a * L + l].size();
+            return w;
+        };
+        std::stable_sort(groups.begin(), groups.end(),
+                         [&](const std::vector<int>& p, const std::vector<int>& q) { return weight(p) > weight(q); });
+        std::vector<int> lout, start(1, 0), item, where(nch, -1);
+        std::vector<float4> csum;
+        coef.clear();
+        for (const auto& g : groups) {
+            lout.insert(lout.end(), g.begin(), g.end());
+            for (int l = 0; l < L; l++) {
+                std::vector<int> bs;
+                for (int a : g)
+                    if (a >= 0)
+                        for (const Use& u : uses[(size_t)a * L + l]) bs.push_back(u.b);
+                std::sort(bs.begin(), bs.end());
+                bs.erase(std::unique(bs.begin(), bs.end()), bs.end());
+                for (int b : bs) {
+                    where[b] = (int)item.size();
+                    item.push_back(b | (B.kap[b] != -1 ? ITEM_NO0 : 0) | (B.kap[b] != 1 ? ITEM_NO1 : 0));
+                }
+                for (; bs.size() % 4; bs.push_back(bs.back())) item.push_back(bs.back());   // padding, used by no output
+                coef.resize(item.size() * no * 4, 0.0);
+                for (int j = 0; j < no; j++) {
+                    double cs[4] = {0, 0, 0, 0};
+                    if (g[j] >= 0)
+                        for (const Use& u : uses[(size_t)g[j] * L + l]) {
+                            const double kb = B.kap[u.b], cv[4] = {u.al, u.al * kb, u.be, u.be * kb};
+                            item[where[u.b]] |= ITEM_USE << j;
+                            for (int k = 0; k < 4; k++) {
+                                coef[((size_t)where[u.b] * no + j) * 4 + k] = cv[k];
+                                cs[k] += std::fabs(cv[k]);
+                            }
+                        }
+                    const double up = 1.0 + 1e-6;
+                    csum.push_back(make_float4((float)(cs[0] * up), (float)(cs[1] * up), (float)(cs[2] * up),
+                                               (float)(cs[3] * up)));
+                }
+                start.push_back((int)item.size());
+            }
+        }
+        int *dout = nullptr, *dstart = nullptr, *di = nullptr;
+        float4* dcs = nullptr;
+        dirac_status e = upload(op, &dout, lout);
+        if (!e) e = upload(op, &dstart, start);
+        if (!e) e = upload(op, &di, item);
+        if (!e) e = upload(op, &dcs, csum);
+        v.L = L; v.nlist = (int)groups.size(); v.out = dout; v.start = dstart; v.item = di; v.csum = dcs;
+        return e;
+    };
+    std::vector<double> coef, coefx;
+    if (!e) e = lists(AG4, op->ang4, coef);
+    const bool mixed = op->opts.precision == 2;   // double-float and complex64 products
+    const size_t ne = (size_t)L * 18 * n1 * 13;   // band entries: 6 sums x 3 values
+    if (mixed) {
+        if (!e) e = lists(AGX, op->angx, coefx);
+        std::vector<float> cf(coef.begin(), coef.end());
+        std::vector<float4> cx(coefx.size());   // each word doubled: the packed operands
+        for (size_t i = 0; i < coefx.size(); i++) {
+            const float h = (float)coefx[i], lo = (float)(coefx[i] - (double)h);
+            cx[i] = make_float4(h, h, lo, lo);
+        }
+        if (!e) e = dev_alloc(op, &op->ang_umax, (size_t)nch * ang_np(n1));
+        if (!e) e = upload(op, &op->ang_c32, cf);
+        if (!e) e = upload(op, &op->ang_cx, cx);
+        AsmSet& a = op->aset[0];
+        if (!e) e = dev_alloc(op, &a.Ef, ne);
+        if (!e) e = dev_alloc(op, &a.Ex, ne);
+        if (!e) e = dev_alloc(op, &a.Ers, (size_t)L * 18 * n1);
+    } else {
+        if (!e) e = upload(op, &op->ang_c64, coef);
+        if (!e) e = dev_alloc(op, &op->Ed, ne);
+    }
+    char* S = nullptr;
+    if (!e) e = dev_alloc(op, &S, ((size_t)nch * (6 * L + (mixed ? 0 : 2)) * ang_np(n1) + ang_tail()) * 16);
+    // where the steps keep the stored form, a card without room for this one still takes the operator
+    if (e == DIRAC_E_NOMEM && mixed && op->opts.tol >= 1e-11) {
+        cudaGetLastError();
+        return DIRAC_OK;
+    }
+    if (e) return e;
+    op->ang_S = S;
+    CUDA_TRY(ang_prepare());
+    op->ang = true;
+    op->ang_step = op->use_ang = ang_steps(op);
+    return DIRAC_OK;
+}
+
 extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dirac_pulse* pulse,
                                              const dirac_solver_opts* opts, void* stream, dirac_op** out)
 {
@@ -863,9 +1110,12 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     TRY(dev_alloc(op, &op->G, (size_t)P.L * 4 * be));
     TRY(dev_alloc(op, &op->s, (size_t)P.L * 3));
     TRY(dev_alloc(op, &op->t_eval, 1));
+    op->pv.L = P.L;
+    if (bd == 13 && op->npairs) TRY(ang_setup(op, ord, kslot));   // factorised products, where they are the faster form
+    const size_t wlen = op->ang_step ? 1 : (size_t)std::max<int64_t>(op->npairs, 1) * be;   // stored coupling values
     if (!dfloat) {
-        TRY(dev_alloc(op, &op->W, (size_t)std::max<int64_t>(op->npairs, 1) * be));
-        TRY(dev_alloc(op, &op->K, (size_t)std::max<size_t>(keyl.size(), 1) * be));
+        TRY(dev_alloc(op, &op->W, wlen));
+        TRY(dev_alloc(op, &op->K, op->ang_step ? 1 : (size_t)std::max<size_t>(keyl.size(), 1) * be));
     } else {
         auto split = [](double v) { float h = (float)v; return make_float2(h, (float)(v - (double)h)); };
         std::vector<float2> sdf(hS.size()), hdf(hH.size());
@@ -948,11 +1198,14 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
             TRY(dev_alloc(op, &op->Kdf, (size_t)std::max<size_t>(keyl.size(), 1) * be));
             TRY(dev_alloc(op, &op->KTdf, (size_t)std::max<size_t>(keyl.size(), 1) * be));
         }
-        TRY(dev_alloc(op, &op->Wh, (size_t)std::max<int64_t>(op->npairs, 1) * be));
-        TRY(dev_alloc(op, &op->Wl, (size_t)std::max<int64_t>(op->npairs, 1) * be));
-        TRY(dev_alloc(op, &op->xsplit, (size_t)op->n));
-        TRY(dev_alloc(op, &op->vsplit, (size_t)op->n));
-        op->aset[0] = AsmSet{op->t_eval, op->s, op->Gdf, op->Kdf, op->KTdf, op->Wh, op->Wl};
+        TRY(dev_alloc(op, &op->Wh, wlen));
+        TRY(dev_alloc(op, &op->Wl, wlen));
+        // split vectors; the factorised form's rows have margins
+        const size_t nsp = std::max((size_t)op->n, (size_t)B.nch * 2 * ang_np(n1) + ang_tail());
+        TRY(dev_alloc(op, &op->xsplit, nsp));
+        TRY(dev_alloc(op, &op->vsplit, nsp));
+        op->aset[0].t_eval = op->t_eval; op->aset[0].s = op->s; op->aset[0].Gdf = op->Gdf;
+        op->aset[0].Kdf = op->Kdf; op->aset[0].KTdf = op->KTdf; op->aset[0].Wh = op->Wh; op->aset[0].Wl = op->Wl;
         op->acur = 0;
     }
 
@@ -961,7 +1214,7 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     op->k64.S = dS; op->k64.H = dH; op->k64.W = op->W; op->k64.U = dU; op->k64.L = dL;
     op->k64.Urow = dUr; op->k64.Dinv = dDi;
     if (mixed) {
-        if (!dfloat) TRY(dev_alloc(op, &op->W32, (size_t)std::max<int64_t>(op->npairs, 1) * be));
+        if (!dfloat) TRY(dev_alloc(op, &op->W32, wlen));
         TRY(alloc_krylov(op, op->k32, 1, opts->tol_inner));
         std::vector<float> fS(hS.begin(), hS.end()), fH(hH.begin(), hH.end());
         auto tof = [](const std::vector<double2>& a) {
@@ -997,6 +1250,18 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
         op->k32.S = fdS; op->k32.H = fdH; op->k32.W = dfloat ? (const void*)op->Wh : (const void*)op->W32;
         op->k32.U = fdU; op->k32.L = fdL;
         if (bd == 13 && op->npairs) {
+            if (dfloat) {
+                TRY(dev_alloc(op, &op->psi32, (size_t)op->n));
+                TRY(dev_alloc(op, &op->b32, (size_t)op->n));
+                TRY(dev_alloc(op, &op->need_b, 1));
+                if (cudaMemsetAsync(op->need_b, 0, sizeof(int), op->st) != cudaSuccess) {
+                    set_error("dirac_operator_setup: cudaMemsetAsync failed");
+                    dirac_op_free(op);
+                    return DIRAC_E_CUDA;
+                }
+            }
+        }
+        if (bd == 13 && op->npairs && !op->ang_step) {
             // partial transposed products of the owner/gather apply
             int ntile = grid_for(n1, apply_own_tile());
             size_t nslot = (size_t)op->npairs * ntile * apply_own_nout();
@@ -1047,14 +1312,6 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
                     }
                     TRY(dev_alloc(op, &op->own_sig, (size_t)op->npairs * ntile * residual_sig_bytes()));
                 }
-                TRY(dev_alloc(op, &op->psi32, (size_t)op->n));
-                TRY(dev_alloc(op, &op->b32, (size_t)op->n));
-                TRY(dev_alloc(op, &op->need_b, 1));
-                if (cudaMemsetAsync(op->need_b, 0, sizeof(int), op->st) != cudaSuccess) {
-                    set_error("dirac_operator_setup: cudaMemsetAsync failed");
-                    dirac_op_free(op);
-                    return DIRAC_E_CUDA;
-                }
             }
             cudaError_t ce = apply_own32_prepare();
             if (ce != cudaSuccess) {
@@ -1070,7 +1327,8 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     op->nparts_prec = grid_for(B.nch, 4);                     // ||s||^2 partials, warp-per-channel kernel
     op->nparts_prec32 = op->prec_warps ? op->prec_warps : grid_for(B.nch, 4);   // lane-per-channel kernel
     int np = std::max({op->nparts_apply, op->nparts_own, op->nparts_vec, op->nparts_prec, op->nparts_prec32,
-                       grid_for(n1, FTR) * B.nch,
+                       grid_for(n1, FTR) * B.nch, op->ang ? rad_parts(0, n1, op->nrad_lanes) : 0,
+                       op->ang ? rad_parts(1, n1, op->nrad_lanes) : 0,
                        precond_sm_blocks<double>(B.nch), precond_sm_blocks<float>(B.nch),
                        precond_rot_blocks<double>(B.nch), precond_rot_blocks<float>(B.nch)});
     TRY(dev_alloc(op, &op->part_d, (size_t)np));
@@ -1142,6 +1400,7 @@ extern "C" dirac_status dirac_apply(dirac_op* op, int sign, double t, const void
     }
     k_set_time<<<1, 1, 0, op->st>>>(op->t_eval, t);
     op->launches++;
+    op->use_ang = op->ang;
     launch_assemble(op);
     apply_accurate(op, sign, x_dev, y_dev, nullptr, nullptr);
     return check_launch("dirac_apply");
@@ -1176,6 +1435,7 @@ extern "C" dirac_status dirac_apply32(dirac_op* op, int sign, double t, const vo
     }
     k_set_time<<<1, 1, 0, op->st>>>(op->t_eval, t);
     op->launches++;
+    op->use_ang = op->ang;
     launch_assemble(op);
     k_apply_launch(op, op->k32, sign, x_dev, y_dev, nullptr, nullptr, nullptr, nullptr, nullptr);
     dirac_status e = check_launch("dirac_apply32");
@@ -1204,12 +1464,13 @@ extern "C" dirac_status dirac_residual(dirac_op* op, double t, const void* psi_d
     Krylov& K = op->k64;
     k_set_time<<<1, 1, 0, op->st>>>(op->t_eval, t);
     op->launches++;
+    op->use_ang = op->ang;
     launch_assemble(op);
     vcopy(op, K, x_dev, K.x);
     // b = A_- psi and ||b||^2 (precision 2 forms both inside the residual pass), then r = b - A_+ x
     if (op->opts.precision == 0) {
         apply_accurate(op, -1, psi_dev, K.b, nullptr, op->part_n);
-        finish(op, K.ks, 0, op->nparts_apply, nullptr, op->part_n, op->opts.max_iter);
+        finish(op, K.ks, 0, apply_parts(op, K), nullptr, op->part_n, op->opts.max_iter);
     } else {
         rhs_accurate(op, psi_dev);
     }
@@ -1236,8 +1497,8 @@ extern "C" dirac_status dirac_op_set_schedule(dirac_op* op, int complex64, int s
     return DIRAC_OK;
 }
 
-// Subgroup form of the factorised apply (mode 1): kappa chunks of up to FLANE channels for the radial
-// pass; for the angular pass, the channels of each mu in FSG-sized subgroups (ordered by the parity
+// Subgroup form of the factorised apply (mode 1): the radial pass takes the kappa chunks of the setup;
+// for the angular pass, the channels of each mu in FSG-sized subgroups (ordered by the parity
 // of their orbital l, then |kappa|, so that a subgroup's outputs share many partners) with the union
 // of their (partner, multipole) items and per item and output the coefficients of U, V, U', V'
 // (own pairs a < b: -(cA, cA ka, cB, cB ka); pairs b < a: (cB, cB ka, cA, cA ka); the apply's sign
@@ -1247,36 +1508,6 @@ static dirac_status fact_sub_setup(dirac_op* op)
     using namespace dg;
     const Basis& B = op->B;
     const int nch = B.nch, L = op->pv.L;
-    // radial: kappa groups of the kappa-sorted channel order, FLANE channels at a time
-    std::vector<int> ks(nch), ordv(nch);
-    CUDA_TRY(cudaMemcpy(ordv.data(), op->ov.prec_order, sizeof(int) * nch, cudaMemcpyDeviceToHost));
-    CUDA_TRY(cudaMemcpy(ks.data(), op->ov.ch_kslot, sizeof(int) * nch, cudaMemcpyDeviceToHost));
-    std::vector<RadChunk> ch1;
-    for (int i = 0; i < nch;) {
-        int j = i;
-        while (j < nch && ks[ordv[j]] == ks[ordv[i]] && j - i < FLANE) j++;
-        ch1.push_back(RadChunk{ks[ordv[i]], B.kap[ordv[i]], i, j - i});
-        i = j;
-    }
-    // two chunks per block where their channels fit the lanes together: largest first, each paired
-    // with the largest unpaired chunk that still fits
-    std::stable_sort(ch1.begin(), ch1.end(), [](const RadChunk& p, const RadChunk& q) { return p.count > q.count; });
-    std::vector<char> used(ch1.size(), 0);
-    std::vector<RadPack> rl;
-    for (size_t i = 0; i < ch1.size(); i++) {
-        if (used[i]) continue;
-        used[i] = 1;
-        RadPack pk{};
-        pk.c[0] = ch1[i];
-        pk.c[1] = RadChunk{ch1[i].ks, ch1[i].kappa, ch1[i].first, 0};
-        for (size_t j = i + 1; j < ch1.size(); j++)
-            if (!used[j] && ch1[i].count + ch1[j].count <= FLANE) {
-                used[j] = 1;
-                pk.c[1] = ch1[j];
-                break;
-            }
-        rl.push_back(pk);
-    }
     // the pair terms' coefficients (cA, cB) = (-c tau A1, c tau A2), from their double-float words
     std::vector<float4> cdf(B.pterm.size());
     if (!cdf.empty())
@@ -1339,12 +1570,10 @@ static dirac_status fact_sub_setup(dirac_op* op)
     // heaviest subgroups first, so the long blocks start in the first wave
     std::stable_sort(subs.begin(), subs.end(), [](const FactSub& p, const FactSub& q) { return p.count > q.count; });
     if (ioff.empty()) { ioff.push_back(0); icoef.assign(FSG, make_float4(0.f, 0.f, 0.f, 0.f)); }
-    dirac_status e = upload(op, &op->rad_lanes, rl);
-    if (!e) e = upload(op, &op->fsub, subs);
+    dirac_status e = upload(op, &op->fsub, subs);
     if (!e) e = upload(op, &op->fitem_off, ioff);
     if (!e) e = upload(op, &op->fitem_coef, icoef);
     if (e) return e;
-    op->nrad_lanes = (int)rl.size();
     op->nfsub = (int)subs.size();
     op->fsub_max = subs.empty() ? 1 : std::max(1, subs[0].count);   // sorted by decreasing count
     CUDA_TRY(fact_sub_prepare(op->fsub_max));
@@ -1375,7 +1604,7 @@ extern "C" dirac_status dirac_op_set_factorised(dirac_op* op, int enable)
         if (e) return e;
         op->nrad = (int)rc.size();
     }
-    if (enable == 1 && !op->fsub) {
+    if (enable == 1 && !op->ang_step && !op->fsub) {
         dirac_status e = fact_sub_setup(op);
         if (e) return e;
         // the G hi words as plain floats, written by every later assembly of each buffer set
@@ -1384,7 +1613,7 @@ extern "C" dirac_status dirac_op_set_factorised(dirac_op* op, int enable)
             if (op->aset[c].Gdf && !op->aset[c].Ghi && (e = dev_alloc(op, &op->aset[c].Ghi, gsz))) return e;
         op->Ghi = op->aset[op->acur].Ghi;
     }
-    if (enable && !op->Zf) {
+    if (enable && !(op->ang_step && enable == 1) && !op->Zf) {
         // products of two radial tiles (the subgroup form forms tile t + 1 while it combines tile t)
         dirac_status e = dev_alloc(op, &op->Zf, (size_t)2 * op->ov.nch * op->pv.L * 4 * FTR * 2);
         if (e) return e;
@@ -1437,7 +1666,7 @@ extern "C" dirac_status dirac_op_set_overlap(dirac_op* op, int enable)
         set_error("dirac_op_set_overlap: bad argument (the overlapped assembly needs precision 2)");
         return DIRAC_E_ARG;
     }
-    if (enable && !op->aset[1].Wh) {
+    if (enable && !op->aset[1].t_eval) {
         size_t be = (size_t)op->ov.n1 * op->ov.bd * 4;
         AsmSet a;
         dirac_status e;
@@ -1445,8 +1674,8 @@ extern "C" dirac_status dirac_op_set_overlap(dirac_op* op, int enable)
             (e = dev_alloc(op, &a.Gdf, (size_t)op->pv.L * 4 * be)) ||
             (!op->asm_chunks && (e = dev_alloc(op, &a.Kdf, (size_t)std::max(op->ov.nkeys, 1) * be))) ||
             (!op->asm_chunks && (e = dev_alloc(op, &a.KTdf, (size_t)std::max(op->ov.nkeys, 1) * be))) ||
-            (e = dev_alloc(op, &a.Wh, (size_t)std::max<int64_t>(op->npairs, 1) * be)) ||
-            (e = dev_alloc(op, &a.Wl, (size_t)std::max<int64_t>(op->npairs, 1) * be)))
+            (e = dev_alloc(op, &a.Wh, op->ang_step ? 1 : (size_t)std::max<int64_t>(op->npairs, 1) * be)) ||
+            (e = dev_alloc(op, &a.Wl, op->ang_step ? 1 : (size_t)std::max<int64_t>(op->npairs, 1) * be)))
             return e;
         CUDA_TRY(cudaStreamCreateWithFlags(&op->st_asm, cudaStreamNonBlocking));
         CUDA_TRY(cudaEventCreateWithFlags(&op->ev_res, cudaEventDisableTiming));
@@ -1455,6 +1684,12 @@ extern "C" dirac_status dirac_op_set_overlap(dirac_op* op, int enable)
             CUDA_TRY(cudaEventCreateWithFlags(&op->ev_use[i], cudaEventDisableTiming));
         }
         if (op->aset[0].Ghi && (e = dev_alloc(op, &a.Ghi, (size_t)op->pv.L * 4 * be))) return e;
+        if (op->ang) {
+            const size_t ne = (size_t)op->pv.L * 18 * op->ov.n1 * 13;
+            if ((e = dev_alloc(op, &a.Ef, ne)) || (e = dev_alloc(op, &a.Ex, ne)) ||
+                (e = dev_alloc(op, &a.Ers, (size_t)op->pv.L * 18 * op->ov.n1)))
+                return e;
+        }
         op->aset[1] = a;
     }
     op->overlap = enable != 0;
@@ -1476,10 +1711,11 @@ extern "C" dirac_status dirac_step(dirac_op* op, void* psi_dev, void* hist_dev, 
     int nh = (hist_dev && n_hist) ? std::max(0, std::min(hmax, *n_hist)) : 0;
     int npv = op->nparts_vec;
     Krylov& K = op->k64;
+    op->use_ang = op->ang_step;
     dirac_status result = DIRAC_OK;
     // overlapped assembly: step s + 1's coupling values are assembled on st_asm into the other buffer
     // set while step s solves; ev_asm[c] marks set c assembled, ev_use[c] the end of its last use
-    const bool ovl = op->overlap && o.precision == 2 && op->aset[1].Wh;
+    const bool ovl = op->overlap && o.precision == 2 && op->aset[1].t_eval;
     const double t_off = o.time_eval ? o.dt : 0.5 * o.dt;
     for (int step = 0; step < n_steps; step++) {
         if (!ovl || step == 0) {
@@ -1509,7 +1745,7 @@ extern "C" dirac_status dirac_step(dirac_op* op, void* psi_dev, void* hist_dev, 
         // b = A_- psi, ||b||^2 (precision 2 forms them inside the residual passes)
         if (o.precision == 0) {
             apply_accurate(op, -1, psi, K.b, nullptr, op->part_n);
-            finish(op, K.ks, 0, op->nparts_apply, nullptr, op->part_n, o.max_iter);
+            finish(op, K.ks, 0, apply_parts(op, K), nullptr, op->part_n, o.max_iter);
         } else {
             rhs_accurate(op, psi);
         }

@@ -103,6 +103,20 @@ struct FactSub {
     int out[FSG];         // output channels (-1: slot unused)
 };
 
+// Factorised apply, angular sums first (kernels_ang.cu): lists of AG4 (or AGX, double-float) output
+// channels of one mu; per (list, multipole) the items start[g L + l] .. are the partners of any of them.
+constexpr int AG4 = 4, AGX = 2;
+constexpr int ITEM_CH = 0xffffff;                            // item word: the partner channel,
+constexpr int ITEM_NO0 = 1 << 24, ITEM_NO1 = 1 << 25;        // its slot-0 function 0, 1 is unused,
+constexpr int ITEM_USE = 1 << 26;                            // bit 26 + j: output j of the list uses it
+struct AngList {
+    int L, nlist;
+    const int* out;           // [nlist][outputs] channels (-1: unused)
+    const int* start;         // [nlist L + 1]; counts are multiples of 4
+    const int* item;          // item words; the coefficients lie apart, [item][outputs][4]
+    const float4* csum;       // [nlist][L][outputs]: sums of |alpha|, |alpha kb|, |beta|, |beta kb| over the items
+};
+
 struct PulseView {
     int L;
     double T, amp, t0, dt;

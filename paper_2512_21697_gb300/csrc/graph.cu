@@ -337,7 +337,7 @@ static dirac_status build_graph(dirac_op* op, GraphDriver* gd, double2* psi, dou
             launch_assemble(op);
             if (o.precision == 0) {
                 apply_accurate(op, -1, psi, K.b, nullptr, op->part_n);
-                finish(op, K.ks, 0, op->nparts_apply, nullptr, op->part_n, o.max_iter);
+                finish(op, K.ks, 0, apply_parts(op, K), nullptr, op->part_n, o.max_iter);
             } else {
                 rhs_accurate(op, psi);
             }
@@ -400,6 +400,7 @@ void graph_free(dirac_op* op)
 // the asynchronous read-back of its results into pinned host memory.  Nothing waits for the GPU.
 dirac_status run_launch(dirac_op* op, double2* psi, double2* h1, int n_hist, int n_steps, double t_start)
 {
+    op->use_ang = op->ang_step;
     if (!op->graph) op->graph = new GraphDriver();
     GraphDriver* gd = op->graph;
     double2* h2 = h1 + op->n;

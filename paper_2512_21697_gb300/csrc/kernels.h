@@ -160,6 +160,33 @@ void launch_fact32_sub(cudaStream_t st, const OpView& A, const RadPack* rl, int 
                        const float* ST, const float* HT, int sign, const void* x, float2* Z, void* y,
                        const void* bsub, const void* dv, double2* pdot, double* pnrm, const KState* skip);
 
+// factorised apply, angular sums first (kernels_ang.cu): two launches per product.  S: workspace of
+// channels x (6 L + 2) x ang_np(n1) + ang_tail() elements (complex64, or 16 bytes; double-float without the + 2);
+// partials: rad_parts slots.
+int ang_np(int n1);
+int ang_tail();
+// split vectors of the double-float product: u = psi + x, v = psi - x (v null: u = psi), channels x 2 x
+// ang_np(n1) + ang_tail() elements each; umax: the largest |u| word per (channel, position)
+void launch_split_rows(cudaStream_t st, int nch, int n1, const double2* psi, const double2* x, float4* u, float4* v,
+                       float2* psi32, float* umax);
+int rad_parts(int prec, int n1, int npack);   // prec 1: complex64, else complex128 / double-float
+cudaError_t ang_prepare();                    // dynamic shared-memory limits (once per device)
+// band entries of the current time factors s in the precisions asked for (null: not), and the
+// double-float ones' row sums
+void launch_rad_entries(cudaStream_t st, const PulseView& P, int n1, const double* s, float* Ef, float2* Ex, double* Ed,
+                        float* rs);
+void launch_ang32(cudaStream_t st, const OpView& A, const AngList& G, const float* coef, const RadPack* rp, int npack,
+                  const float* E, const float* Sb, const float* Hb, int sign, const void* x, void* S, void* y,
+                  const void* bsub, const void* dv, double2* pdot, double* pnrm, const KState* skip, const int* gate);
+void launch_ang64(cudaStream_t st, const OpView& A, const AngList& G, const double* coef, const RadPack* rp, int npack,
+                  const double* E, const double* Sb, const double* Hb, int sign, const void* x, void* S, void* y,
+                  const void* bsub, const void* dv, double2* pdot, double* pnrm, const KState* skip);
+// y = Sb v + sign (i Ht u + coupling u) in double-float from type-major split vectors u, v (offsets: the
+// fixed-binade accumulators, else Dot2); with v = psi - x, u = psi + x and sign -1 the refinement residual
+void launch_ang_df(cudaStream_t st, const OpView& A, const AngList& G, bool offsets, const float4* coef,
+                   const RadPack* rp, int npack, const float2* E, const float* rs, const float2* Sb, const float2* Ht,
+                   int sign, const float4* u, const float* umax, const float4* v, void* S, double2* y, double* pnrm);
+
 // learned-guess network forward on the fifth-generation tensor cores (tcgen05, TMEM accumulators)
 size_t guess_forward_tc05_smem();
 int64_t guess_tc05_packed();

@@ -35,6 +35,11 @@ struct AsmSet {
     float2 *Gdf = nullptr, *Kdf = nullptr, *KTdf = nullptr;
     float *Wh = nullptr, *Wl = nullptr;
     float* Ghi = nullptr;   // hi words of Gdf as plain floats (factorised apply, subgroup form)
+    // band entries of the factorised products at this time (kernels_ang.cu): complex64, double-float and
+    // the double-float ones' row sums
+    float* Ef = nullptr;
+    float2* Ex = nullptr;
+    float* Ers = nullptr;
 };
 
 }  // namespace dg
@@ -79,12 +84,24 @@ struct dirac_op {
     int fact32 = 0;              // 0 stored coupling, 1 subgroup form, 2 per-channel form
     dg::RadChunk* rad_chunks = nullptr;
     int nrad = 0;
-    dg::RadPack* rad_lanes = nullptr;    // subgroup form: pairs of kappa chunks sharing FLANE lanes
+    dg::RadPack* rad_lanes = nullptr;    // pairs of kappa chunks sharing FLANE lanes
     int nrad_lanes = 0;
     dg::FactSub* fsub = nullptr;         // subgroup form: FSG outputs of one mu and their items
     int nfsub = 0, fsub_max = 1;         // subgroups, the largest item count
     int* fitem_off = nullptr;            // item -> partner * L + multipole
     float4* fitem_coef = nullptr;        // item -> FSG coefficient sets (U, V, U', V')
+    // factorised products with the angular sums first (kernels_ang.cu), the accurate and the complex64
+    // ones, for systems where they are the faster form
+    bool ang = false;                    // they are set up: single products take them
+    bool ang_step = false;               // steps take them, too: no coupling values are stored
+    bool use_ang = false;                // the form of the running call, and of the last assembly
+    dg::AngList ang4{}, angx{};          // lists of AG4 and of AGX outputs
+    float* ang_c32 = nullptr;            // angular coefficients of the items in each precision in use
+    float4* ang_cx = nullptr;
+    double* ang_c64 = nullptr;
+    void* ang_S = nullptr;               // the angular sums of one apply
+    float* ang_umax = nullptr;           // largest |u| per position (double-float)
+    double* Ed = nullptr;                // FP64 band entries (precision 0 and 1)
     float2* Zf = nullptr;        // band products of one radial tile
     float* Ghi = nullptr;        // the current buffer set's G hi words (subgroup form)
     // grouped double-float assembly (null when a group has more than ASM_MAX_NL multipoles)
