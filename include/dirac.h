@@ -332,9 +332,9 @@ dirac_status dirac_op_set_residual_mode(dirac_op* op, int mode);
 /* Preconditioner schedule of the complex128 (complex64 = 0) or complex64 (complex64 = 1) solve:
  * 0 one lane per channel (complex64 only; the channels of one kappa share the factor rows),
  * 1 one warp per channel, 2 one warp per channel with the vector and the factor rows staged
- * through shared memory, 3 one warp per channel with each row fixed to one lane (one shuffle
- * round per row; only factor chunks in shared memory, so every channel's warp is resident at
- * once).  dirac_operator_setup times the available ones and keeps the fastest; this call
+ * through shared memory, 3 sixteen lanes per channel (32 where the factors' interchanges reach
+ * further than two rows) with each row fixed to one lane (one shuffle round per row; the factors
+ * in registers, so every channel is resident at once).  dirac_operator_setup times the available ones and keeps the fastest; this call
  * overrides it (DIRAC_E_ARG if the schedule is not available for the op).  Schedules 1, 2 and 3
  * perform the same operations in the same order; 0 rounds differently (within the solver
  * tolerance). */

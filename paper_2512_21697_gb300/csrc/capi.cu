@@ -353,7 +353,7 @@ void k_precond_launch(dirac_op* op, const Krylov& K, int mode, const KState* ks,
         else if (op->prec_sched32 == 2 && op->prec_sm_ok)
             launch_precond_sm_t<float>(op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z, pn);
         else if (op->prec_sched32 == 3 && op->prec_rot_ok)
-            launch_precond_rot_t<float>(op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z, pn);
+            launch_precond_rot_t<float>(op->st, op->ov, op->rot_lanes, K.rotF, K.rotB, K.Dinv, op->rot_piv, mode, ks, r, v, io, z, pn);
         else
             launch_precond_t<float>(grid_for(op->ov.nch, 4), op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z,
                                     pn);
@@ -361,7 +361,7 @@ void k_precond_launch(dirac_op* op, const Krylov& K, int mode, const KState* ks,
         if (op->prec_sched64 == 2 && op->prec_sm_ok)
             launch_precond_sm_t<double>(op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z, pn);
         else if (op->prec_sched64 == 3 && op->prec_rot_ok)
-            launch_precond_rot_t<double>(op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z, pn);
+            launch_precond_rot_t<double>(op->st, op->ov, op->rot_lanes, K.rotF, K.rotB, K.Dinv, op->rot_piv, mode, ks, r, v, io, z, pn);
         else
             launch_precond_t<double>(grid_for(op->ov.nch, 4), op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z,
                                      pn);
@@ -1071,13 +1071,58 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
             hL[(size_t)ks * ns * kb + e] = make_double2(lu.L[e].real(), lu.L[e].imag());
         std::copy(lu.piv.begin(), lu.piv.end(), hP.begin() + (size_t)ks * ns);
     }
+    // in FP64 the warp schedules take U's rows divided by their diagonals (column form)
+    auto by_diag = [&](int ks, int i, int k) {
+        const size_t e = ((size_t)ks * ns + i) * (wu + 1) + k;
+        const cd u = i - k >= 0 ? cd(hU[e].x, hU[e].y) * cd(hDi[(size_t)ks * ns + i - k].x, hDi[(size_t)ks * ns + i - k].y)
+                                : cd(0);
+        return make_double2(u.real(), u.imag());
+    };
+    std::vector<double2> hUs(hU.size());
+    for (int ks = 0; ks < nk2; ks++)
+        for (int i = 0; i < ns; i++)
+            for (int k = 0; k <= wu; k++) hUs[((size_t)ks * ns + i) * (wu + 1) + k] = by_diag(ks, i, k);
     double2 *dU, *dL, *dUr, *dDi;
     int *dP, *dord;
-    TRY(upload(op, &dU, hU));
+    TRY(upload(op, &dU, hUs));
     TRY(upload(op, &dL, hL));
     TRY(upload(op, &dUr, hUr));
     TRY(upload(op, &dDi, hDi));
     TRY(upload(op, &dP, hP));
+    // the rotated-lane schedule's tables, entry (row, lane): forward the multiplier of the row that the
+    // lane holds (row + 1 .. row + kb), backward 1 / U[i][i] in row i's lane and U[i - m][i] in row i - m's;
+    // zero elsewhere.  16 lanes hold the backward window if U's superdiagonals from 16 on are zero.
+    std::vector<double2> hRF, hRB;
+    double2 *dRF = nullptr, *dRB = nullptr;
+    if (bd == 13) {
+        int W = 16;
+        for (size_t e = 0; e < hU.size(); e++)
+            if (e % (wu + 1) >= 16 && (hU[e].x != 0 || hU[e].y != 0)) W = 32;
+        const size_t np = (size_t)(ns + W - 1) / W * W;
+        hRF.assign(nk2 * np * W, make_double2(0, 0));
+        hRB = hRF;
+        std::vector<unsigned char> pl(nk2 * np);
+        for (int ks = 0; ks < nk2; ks++)
+            for (size_t j = 0; j < np; j++) {
+                const size_t row = ks * np + j, s = (size_t)ks * ns + j;
+                pl[row] = (unsigned char)((j < (size_t)ns ? hP[s] : (int)j) % W);
+                if (j >= (size_t)ns) continue;
+                for (int k = 1; k <= kb && j + k < (size_t)ns; k++) hRF[row * W + (j + k) % W] = hL[s * kb + k - 1];
+                hRB[row * W + j % W] = hDi[s];
+                for (int m = 1; m < W && m <= wu && (size_t)m <= j; m++)
+                    hRB[row * W + (j - m) % W] = hU[s * (wu + 1) + m];
+            }
+        std::vector<double2> hRBs(hRB.size(), make_double2(0, 0));   // in FP64, without the diagonal
+        for (size_t row = 0; row < nk2 * np; row++)
+            for (size_t j = row % np, m = 1; j < (size_t)ns && m < (size_t)W && m <= (size_t)wu && m <= j; m++)
+                hRBs[row * W + (j - m) % W] = hUs[(row / np * ns + j) * (wu + 1) + m];
+        op->rot_lanes = W;
+        TRY(upload(op, &dRF, hRF));
+        TRY(upload(op, &dRB, hRBs));
+        std::vector<uint4> pv(pl.size() / 16);
+        std::memcpy(pv.data(), pl.data(), pl.size());
+        TRY(upload(op, &op->rot_piv, pv));
+    }
     std::vector<int> ord(B.nch);
     for (int a = 0; a < B.nch; a++) ord[a] = a;
     std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return kslot[x] < kslot[y]; });
@@ -1213,6 +1258,7 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     TRY(alloc_krylov(op, op->k64, 0, opts->tol));
     op->k64.S = dS; op->k64.H = dH; op->k64.W = op->W; op->k64.U = dU; op->k64.L = dL;
     op->k64.Urow = dUr; op->k64.Dinv = dDi;
+    op->k64.rotF = dRF; op->k64.rotB = dRB;
     if (mixed) {
         if (!dfloat) TRY(dev_alloc(op, &op->W32, wlen));
         TRY(alloc_krylov(op, op->k32, 1, opts->tol_inner));
@@ -1247,6 +1293,12 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
         TRY(upload(op, &fdUr, fUr));
         TRY(upload(op, &fdDi, fDi));
         op->k32.Urow = fdUr; op->k32.Dinv = fdDi;
+        if (bd == 13) {
+            float2 *fRF, *fRB;
+            TRY(upload(op, &fRF, tof(hRF)));
+            TRY(upload(op, &fRB, tof(hRB)));
+            op->k32.rotF = fRF; op->k32.rotB = fRB;
+        }
         op->k32.S = fdS; op->k32.H = fdH; op->k32.W = dfloat ? (const void*)op->Wh : (const void*)op->W32;
         op->k32.U = fdU; op->k32.L = fdL;
         if (bd == 13 && op->npairs) {
@@ -1373,9 +1425,7 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     op->prec_sm_ok = bd == 13 && precond_sm_prepare<float>(n1) == cudaSuccess &&
                      precond_sm_prepare<double>(n1) == cudaSuccess;
     cudaGetLastError();
-    op->prec_rot_ok = bd == 13 && precond_rot_prepare<float>() == cudaSuccess &&
-                      precond_rot_prepare<double>() == cudaSuccess;
-    cudaGetLastError();
+    op->prec_rot_ok = bd == 13;
     {
         dirac_status ts = tune_precond(op, op->k64);
         if (!ts && mixed) ts = tune_precond(op, op->k32);

@@ -137,12 +137,12 @@ template <class T>
 void launch_precond_sm_t(cudaStream_t st, const OpView& A, const void* U, const void* L, const void* Dinv, int mode,
                          const KState* ks, const void* r, const void* v, void* io, void* z, double* pn);
 
-// rotated-lane warp-per-channel preconditioner (band width 13): factor chunks only in shared memory
-template <class T> cudaError_t precond_rot_prepare();
+// rotated-lane preconditioner (band width 13), 16 or 32 lanes per channel; F, Bk, piv: its factor tables
+// [kappa slot][row, padded to a multiple of lanes][lane] and pivot lanes [kappa slot][row]
 template <class T> int precond_rot_blocks(int nch);
 template <class T>
-void launch_precond_rot_t(cudaStream_t st, const OpView& A, const void* U, const void* L, const void* Dinv, int mode,
-                          const KState* ks, const void* r, const void* v, void* io, void* z, double* pn);
+void launch_precond_rot_t(cudaStream_t st, const OpView& A, int lanes, const void* F, const void* Bk,
+                          const void* Dinv, const uint4* piv, int mode, const KState* ks, const void* r, const void* v, void* io, void* z, double* pn);
 
 // bounded-wait self-test: one block waits `limit` cycles on an mbarrier nothing completes
 cudaError_t launch_wait_selftest(cudaStream_t st, long long limit, int* err);

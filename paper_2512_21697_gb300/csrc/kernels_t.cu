@@ -22,6 +22,13 @@ template <class T> __device__ __forceinline__ c2<T> cdv(c2<T> a, c2<T> b)
     T d = b.x * b.x + b.y * b.y;
     return mk<T>((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
 }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+// a b with its roundings fixed
+template <class T> __device__ __forceinline__ c2<T> cm_pin(c2<T> a, c2<T> b)
+{
+    return mk<T>(fma(a.x, b.x, -rmul(a.y, b.y)), fma(a.y, b.x, rmul(a.x, b.y)));
+}
 template <class T> __device__ __forceinline__ c2<T> from_d(double2 a) { return mk<T>((T)a.x, (T)a.y); }
 
 // ---------------------------------------------------------------------------------------------
@@ -175,6 +182,48 @@ __device__ __forceinline__ c2<T> shfl2_down(c2<T> v, int d)
     return mk<T>(__shfl_down_sync(0xffffffffu, v.x, d), __shfl_down_sync(0xffffffffu, v.y, d));
 }
 
+// The steps of the warp schedules' substitutions.  The FP64 unit is narrow and slow to answer on this part
+// (a warp's operation takes it 16 cycles, a dependent one about 40), so in double a step is four
+// multiply-adds, two of them dependent: b - l z directly, and backward the remainder of a row, which starts
+// from z[i] / U[i][i] (pre_scale, off the chain) and ends as x[i], U's rows having been divided by their
+// diagonals at setup.  In float the rounding of the products comes first, as in the lane-per-channel form.
+template <class T>
+__device__ __forceinline__ void sub_prod(c2<T>& w, c2<T> l, c2<T> z)
+{
+    if constexpr (sizeof(T) == 8) {
+        w.x = fma(l.y, z.y, fma(-l.x, z.x, w.x));
+        w.y = fma(-l.y, z.x, fma(-l.x, z.y, w.y));
+    } else {
+        w.x -= l.x * z.x - l.y * z.y;
+        w.y -= l.x * z.y + l.y * z.x;
+    }
+}
+// backward: acc is the remainder of a row (double), or the sum of its products so far (float)
+template <class T>
+__device__ __forceinline__ void add_back(c2<T>& acc, c2<T> u, c2<T> x)
+{
+    if constexpr (sizeof(T) == 8) {
+        sub_prod<T>(acc, u, x);
+    } else {
+        acc.x += u.x * x.x - u.y * x.y;
+        acc.y += u.x * x.y + u.y * x.x;
+    }
+}
+template <class T>
+__device__ __forceinline__ void pre_scale(c2<T>* z, const c2<T>* D, int n, int lane)
+{
+    if constexpr (sizeof(T) == 8) {
+        for (int i = lane; i < n; i += 32) z[i] = cm_pin<T>(z[i], D[i]);
+        __syncwarp();
+    }
+}
+// the accumulator of a row that enters the backward window
+template <class T>
+__device__ __forceinline__ c2<T> back_start(const c2<T>* z, int row)
+{
+    return sizeof(T) == 8 && row >= 0 ? z[row] : mk<T>(0, 0);
+}
+
 template <class T>
 __global__ void __launch_bounds__(128) k_precond(OpView A, const c2<T>* __restrict__ Ucol,
                                                  const c2<T>* __restrict__ L, const c2<T>* __restrict__ Dinv,
@@ -234,8 +283,7 @@ __global__ void __launch_bounds__(128) k_precond(OpView A, const c2<T>* __restri
             else if (lane == pj) w = w0;
             c2<T> zj = shfl2<T>(w, 0);
             if (lane >= 1 && lane <= kb && j + lane < n) {
-                w.x -= lcur.x * zj.x - lcur.y * zj.y;
-                w.y -= lcur.x * zj.y + lcur.y * zj.x;
+                sub_prod<T>(w, lcur, zj);
             }
             if (lane == 0) zc[j] = zj;
             w = shfl2_down<T>(w, 1);
@@ -244,7 +292,8 @@ __global__ void __launch_bounds__(128) k_precond(OpView A, const c2<T>* __restri
         __syncwarp();
         // backward: lane k (1..wu) holds the partial sum of row i - k; the row of U for the next
         // step is loaded one step ahead
-        c2<T> acc = mk<T>(0, 0);
+        pre_scale<T>(zc, Dk, n, lane);
+        c2<T> acc = lane >= 1 && lane <= wu ? back_start<T>(zc, n - lane) : mk<T>(0, 0);
         c2<T> unext = (lane >= 1 && lane <= wu && n - 1 - lane >= 0) ? Uk[(int64_t)(n - 1) * (wu + 1) + lane]
                                                                       : mk<T>(0, 0);
         for (int i = n - 1; i >= 0; i--) {
@@ -256,17 +305,14 @@ __global__ void __launch_bounds__(128) k_precond(OpView A, const c2<T>* __restri
             c2<T> xi = mk<T>(0, 0);
             if (lane == 0) {
                 c2<T> zi = zc[i];
-                xi = cm<T>(mk<T>(zi.x - a0.x, zi.y - a0.y), Dk[i]);
+                xi = sizeof(T) == 8 ? a0 : cm<T>(mk<T>(zi.x - a0.x, zi.y - a0.y), Dk[i]);
                 zc[i] = xi;
             }
             xi = shfl2<T>(xi, 0);
             // slide: lane k takes the sum of row (i-1) - k from lane k + 1, then adds U[i-k][k] x[i]
             acc = shfl2_down<T>(acc, 1);
-            if (lane == wu) acc = mk<T>(0, 0);
-            if (lane >= 1 && lane <= wu) {
-                acc.x += ucur.x * xi.x - ucur.y * xi.y;
-                acc.y += ucur.x * xi.y + ucur.y * xi.x;
-            }
+            if (lane == wu) acc = back_start<T>(zc, i - wu);
+            if (lane >= 1 && lane <= wu) add_back<T>(acc, ucur, xi);
         }
     }
     if (part_nrm) {
@@ -561,8 +607,7 @@ __global__ void k_precond_sm(OpView A, const c2<T>* __restrict__ Ucol, const c2<
                 else if (lane == pj) w = w0;
                 c2<T> zj = shfl2<T>(w, 0);
                 if (lane >= 1 && lane <= KB && j + lane < n) {
-                    w.x -= lcur.x * zj.x - lcur.y * zj.y;
-                    w.y -= lcur.x * zj.y + lcur.y * zj.x;
+                    sub_prod<T>(w, lcur, zj);
                 }
                 if (lane == 0) zs[j] = zj;
                 w = shfl2_down<T>(w, 1);
@@ -578,7 +623,8 @@ __global__ void k_precond_sm(OpView A, const c2<T>* __restrict__ Ucol, const c2<
             cp_async_commit();
         };
         issue_bwd(nc - 1, 0);
-        c2<T> acc = mk<T>(0, 0);
+        pre_scale<T>(zs, Dk, n, lane);
+        c2<T> acc = lane >= 1 && lane <= WU ? back_start<T>(zs, n - lane) : mk<T>(0, 0);
         for (int q = 0; q < nc; q++) {
             const int c = nc - 1 - q;
             if (c > 0) {
@@ -598,16 +644,13 @@ __global__ void k_precond_sm(OpView A, const c2<T>* __restrict__ Ucol, const c2<
                 c2<T> xi = mk<T>(0, 0);
                 if (lane == 0) {
                     c2<T> zi = zs[i];
-                    xi = cm<T>(mk<T>(zi.x - a0.x, zi.y - a0.y), Dc[ii]);
+                    xi = sizeof(T) == 8 ? a0 : cm<T>(mk<T>(zi.x - a0.x, zi.y - a0.y), Dc[ii]);
                     zs[i] = xi;
                 }
                 xi = shfl2<T>(xi, 0);
                 acc = shfl2_down<T>(acc, 1);
-                if (lane == WU) acc = mk<T>(0, 0);
-                if (lane >= 1 && lane <= WU) {
-                    acc.x += ucur.x * xi.x - ucur.y * xi.y;
-                    acc.y += ucur.x * xi.y + ucur.y * xi.x;
-                }
+                if (lane == WU) acc = back_start<T>(zs, i - WU);
+                if (lane >= 1 && lane <= WU) add_back<T>(acc, ucur, xi);
             }
             __syncwarp();
         }
@@ -619,214 +662,209 @@ __global__ void k_precond_sm(OpView A, const c2<T>* __restrict__ Ucol, const c2<
 }
 
 // ---------------------------------------------------------------------------------------------
-// Rotated-lane form of the same substitutions: row r of the window lives in lane r mod 32 for
-// its whole life, so the window never shifts.  A forward step j takes the pivot row's value with
-// one shuffle (plus the row-j value for the interchange, in parallel), and the lanes of rows
-// j+1..j+kb subtract L[j] z[j]; a backward step i forms x[i] in lane i mod 32 from its completed
-// sum and broadcasts it with one shuffle to the lanes of rows i-1..i-2kb.  That is one shuffle
-// round per row on the dependency chain (two in the shifting window).  The vector never lives
-// whole in shared memory: 16-row chunks of the input (forward) and of the forward result
-// (backward) arrive by cp.async together with the factor chunks, so a warp needs a few KB and
-// every channel's warp is resident at once.  The forward result goes to z and comes back for the
-// backward sweep.  Same arithmetic, in the same order, as the shifting-window kernels.
+// Rotated-lane form of the same substitutions: W lanes per channel, row r of the window in lane r mod W
+// for its whole life, so the window never shifts.  A forward step j takes the pivot row's value with
+// one shuffle round (plus the row-j value for the interchange, in parallel) and the lanes of rows
+// j+1..j+kb subtract L[j] z[j]; a backward step i forms x[i] in lane i mod W from its completed sum
+// and broadcasts it to the lanes of the rows above.  A lane that is done with its row keeps the result
+// for one store per W rows and takes the row W further on, which was loaded a chunk before; in modes 1
+// and 2 the input vector is formed at that point.
+//
+// Bound by latency: 2 x 2 n1 dependent steps, of which this form leaves the shuffle and three (forward)
+// or six (backward) dependent operations.  So the factors come in an order of their own, one entry per
+// lane and step (rot_tables: zero outside the window, the diagonal's reciprocal in the finished row's
+// lane): no predicates, no address arithmetic, one load of a register that is used a chunk later.
+// With the interchanges reaching at most two rows (S + i tau H0 at every step size in use) U has 15
+// superdiagonals that are not zero, so W = 16 lanes hold both windows and a warp takes two channels;
+// W = 32 serves factors whose interchanges reach further.  A chunk's factors are asked for from memory four
+// chunks ahead (between two applications the solve streams more than L2 holds).  Same arithmetic, in the
+// same order, as the shifting-window kernels.
+// Against one channel per warp with the factors staged in shared memory, at 1001 slots: complex64 422 -> 202
+// us for 12 channels, 596 -> 285 us for 1860 (factors from memory; 348 without asking ahead); complex128
+// (and the shorter steps of sub_prod) 1475 -> 801 us for 12 channels, 3836 -> 924 us for 1624.
 // ---------------------------------------------------------------------------------------------
 template <class T>
-constexpr int prec_rot_warps() { return sizeof(T) == 4 ? 4 : 2; }
+__host__ __device__ constexpr int rot_cpb() { return sizeof(T) == 4 ? 4 : 2; }   // channels per block (one partial of ||s||^2)
 
-constexpr int ROT_VRING = 4;   // vector chunks in flight per warp (forward input, backward z)
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-template <class T, int KB>
-__host__ __device__ constexpr size_t prec_rot_warp_bytes()
+template <class T, int W>
+__global__ void __launch_bounds__(rot_cpb<T>() * W) k_precond_rot(
+    OpView A, const c2<T>* __restrict__ F, const c2<T>* __restrict__ Bk, const c2<T>* __restrict__ Dinv,
+    const uint4* __restrict__ piv, int mode, const KState* st, const c2<T>* __restrict__ r, const c2<T>* __restrict__ v, c2<T>* __restrict__ io,
+    c2<T>* __restrict__ z, double* part_nrm)
 {
-    return prec_sm_fbytes<T, KB>() + sizeof(c2<T>) * ROT_VRING * PCH;
-}
-
-template <class T, int KB>
-__global__ void k_precond_rot(OpView A, const c2<T>* __restrict__ Ucol, const c2<T>* __restrict__ L,
-                              const c2<T>* __restrict__ Dinv, int mode, const KState* st,
-                              const c2<T>* __restrict__ r, const c2<T>* __restrict__ v, c2<T>* __restrict__ io,
-                              c2<T>* __restrict__ z, double* part_nrm)
-{
-    constexpr int WU = 2 * KB;
-    static_assert(WU + 1 <= 32 && KB < PCH, "the windows must fit in a warp and reach one chunk ahead");
-    extern __shared__ __align__(16) unsigned char prec_smem[];
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int warp = blockIdx.x * (blockDim.x >> 5) + wib;
-    const int n = 2 * A.n1;
-    unsigned char* fb = prec_smem + (size_t)wib * prec_rot_warp_bytes<T, KB>();
-    c2<T>* Lb = reinterpret_cast<c2<T>*>(fb);                          // [2][PCH * KB]
-    int* Pb = reinterpret_cast<int*>(fb + sizeof(c2<T>) * 2 * PCH * KB);  // [2][PCH]
-    c2<T>* Ub = reinterpret_cast<c2<T>*>(fb);                          // [2][PCH * (WU + 1)]
-    c2<T>* Db = Ub + 2 * PCH * (WU + 1);                               // [2][PCH]
-    c2<T>* Vb = reinterpret_cast<c2<T>*>(fb + prec_sm_fbytes<T, KB>());  // [ROT_VRING][PCH]
-    double nsum = 0;
-    if (warp < A.nch && !(st && st->done)) {
-        const int ch = A.prec_order[warp];
-        const int ks = A.ch_kslot[ch];
-        const c2<T>* Uk = Ucol + (int64_t)ks * n * (WU + 1);
-        const c2<T>* Lk = L + (int64_t)ks * n * KB;
-        const c2<T>* Dk = Dinv + (int64_t)ks * n;
-        const int* P = A.luP + (int64_t)ks * n;
+    constexpr int CPB = rot_cpb<T>(), AHEAD = 4;
+    const int l = threadIdx.x % W, slot = threadIdx.x / W, pos = blockIdx.x * CPB + slot;
+    const int n = 2 * A.n1, nc = (n + W - 1) / W;
+    const bool ok = pos < A.nch;
+    double n0 = 0, n1 = 0;   // ||s||^2 of the rows r with r mod 32 < 16, and of the others (W = 32: all in n0)
+    // a warp's first channel decides whether it has work (uniform over the warp)
+    const bool work = blockIdx.x * CPB + (threadIdx.x & ~31) / W < A.nch;
+    if (work && !(st && st->done)) {
+        const int ch = A.prec_order[ok ? pos : A.nch - 1];
+        const int64_t tab = (int64_t)A.ch_kslot[ch] * nc;   // chunks before this kappa's
+        const c2<T>* Fp = F + tab * (W * W) + l;
+        const c2<T>* Bp = Bk + tab * (W * W) + l;
+        const c2<T>* Dp = Dinv + (int64_t)A.ch_kslot[ch] * n;
+        const uint4* Pp = piv + tab * (W / 16);
         const int64_t o = (int64_t)ch * n;
-        // prologue: the input vector, in global memory
-        const c2<T>* b = r + o;
-        if (mode == 1) {
-            c2<T> beta = from_d<T>(st->beta), omega = from_d<T>(st->omega);
-            for (int i = lane; i < n; i += 32) {
-                c2<T> pv = io[o + i], vv = v[o + i], rv = r[o + i];
-                c2<T> t = cm<T>(omega, vv);
-                c2<T> q = cm<T>(beta, mk<T>(pv.x - t.x, pv.y - t.y));
-                io[o + i] = mk<T>(rv.x + q.x, rv.y + q.y);
-            }
-            b = io + o;
-        } else if (mode == 2) {
-            c2<T> alpha = from_d<T>(st->alpha);
-            for (int i = lane; i < n; i += 32) {
-                c2<T> t = cm<T>(alpha, v[o + i]);
-                c2<T> rv = r[o + i];
-                c2<T> sv = mk<T>(rv.x - t.x, rv.y - t.y);
-                io[o + i] = sv;
-                nsum += (double)sv.x * sv.x + (double)sv.y * sv.y;
-            }
-            b = io + o;
-        }
-        __syncwarp();   // the prologue's stores are visible to the warp's copies below
         c2<T>* zo = z + o;
-        const int nc = (n + PCH - 1) / PCH;
-        auto copy_vec = [&](const c2<T>* src, int c) {   // vector chunk c (rows < n) into its ring slot
-            int j0 = c * PCH, rows = min(PCH, n - j0);
-            if (rows > 0) warp_copy16(Vb + (c % ROT_VRING) * PCH, src + j0, rows * (int)sizeof(c2<T>), lane);
+        c2<T> c1 = mk<T>(0, 0), c3 = mk<T>(0, 0);
+        if (mode == 1) { c1 = from_d<T>(st->beta); c3 = from_d<T>(st->omega); }
+        if (mode == 2) c1 = from_d<T>(st->alpha);
+        struct Raw { c2<T> r, v, p; };
+        auto load = [&](int row) {
+            Raw a = {mk<T>(0, 0), mk<T>(0, 0), mk<T>(0, 0)};
+            if (ok && row < n) {
+                a.r = r[o + row];
+                if (mode) a.v = v[o + row];
+                if (mode == 1) a.p = io[o + row];
+            }
+            return a;
         };
-        // forward group c: factor chunk c and input chunk c + 1 (input chunk 0 goes with group 0)
-        auto issue_fwd = [&](int c, int bb) {
-            int j0 = c * PCH, rows = min(PCH, n - j0);
-            warp_copy16(Lb + bb * PCH * KB, Lk + (int64_t)j0 * KB, rows * KB * (int)sizeof(c2<T>), lane);
-            for (int e = lane; e < rows; e += 32) cp_async4(Pb + bb * PCH + e, P + j0 + e);
-            if (c == 0) copy_vec(b, 0);
-            copy_vec(b, c + 1);
-            cp_async_commit();
+        // (the products rounded as in the other schedules' loops)
+        auto input = [&](const Raw& a, int row) {   // the input vector's entry of a row
+            if (mode == 0) return a.r;
+            const bool in = ok && row < n;
+            if (mode == 1) {
+                const c2<T> t = cm_pin<T>(c3, a.v), s = mk<T>(a.p.x - t.x, a.p.y - t.y);
+                const c2<T> b = mk<T>(a.r.x + fma(c1.x, s.x, -rmul(c1.y, s.y)), a.r.y + fma(c1.x, s.y, rmul(c1.y, s.x)));
+                if (in) io[o + row] = b;
+                return b;
+            }
+            const c2<T> t = cm_pin<T>(c1, a.v), sv = mk<T>(a.r.x - t.x, a.r.y - t.y);
+            if (in) {
+                io[o + row] = sv;
+                if (W == 16 && (row & 16)) n1 += (double)sv.x * sv.x + (double)sv.y * sv.y;
+                else n0 += (double)sv.x * sv.x + (double)sv.y * sv.y;
+            }
+            return sv;
         };
-        issue_fwd(0, 0);
-        // forward: lane l holds row j + ((l - j) mod 32); rows j .. j + KB form the window
-        c2<T> w = mk<T>(0, 0);
+        // the factor entries of a chunk on their way into L2 AHEAD chunks before they are loaded
+        auto fetch = [&](const c2<T>* tp, int c) {
+            if (c < 0 || c >= nc) return;
+            constexpr int LINE = 128 / (int)sizeof(c2<T>);
+#pragma unroll
+            for (int e = 0; e < W * W / LINE; e += W)
+                if (e + l < W * W / LINE) prefetch_l2(tp - l + (int64_t)c * (W * W) + (e + l) * LINE);
+        };
+        for (int c = 1; c < AHEAD; c++) fetch(Fp, c);
+        c2<T> f[W];
+#pragma unroll
+        for (int jj = 0; jj < W; jj++) f[jj] = Fp[jj * W];
+        unsigned pq[W / 4];
+        auto pivots = [&](int c, unsigned* q) {
+#pragma unroll
+            for (int e = 0; e < W / 16; e++) {
+                const uint4 p = Pp[c * (W / 16) + e];
+                q[4 * e] = p.x; q[4 * e + 1] = p.y; q[4 * e + 2] = p.z; q[4 * e + 3] = p.w;
+            }
+        };
+        pivots(0, pq);
+        c2<T> w = input(load(l), l), wn = input(load(W + l), W + l), out = mk<T>(0, 0);
         for (int c = 0; c < nc; c++) {
-            if (c + 1 < nc) {
-                issue_fwd(c + 1, (c + 1) & 1);
-                cp_async_wait1();
-            } else {
-                cp_async_wait0();
+            const Raw nxt = load((c + 2) * W + l);
+            const c2<T> di = sizeof(T) == 8 && c * W + l < n ? Dp[c * W + l] : mk<T>(0, 0);
+            fetch(Fp, c + AHEAD);
+            if (l == 0 && ok && (c + AHEAD) * W < n) {
+                const int64_t e = o + (c + AHEAD) * W;
+                prefetch_l2(r + e);
+                if (mode) prefetch_l2(v + e);
+                if (mode == 1) prefetch_l2(io + e);
             }
-            __syncwarp();
-            if (c == 0 && lane < KB && lane < n) w = Vb[lane];   // rows 0 .. KB - 1 start the window
-            const c2<T>* Lc = Lb + (c & 1) * PCH * KB;
-            const int* Pc = Pb + (c & 1) * PCH;
-            const int j0 = c * PCH, rows = min(PCH, n - j0);
+            unsigned pn[W / 4];
+            pivots(min(c + 1, nc - 1), pn);
+            const c2<T>* Fn = Fp + (int64_t)min(c + 1, nc - 1) * (W * W);
 #pragma unroll
-            for (int jj = 0; jj < PCH; jj++) {
-                if (jj >= rows) break;
-                const int j = j0 + jj;
-                const int k = (lane - j) & 31;   // this lane's row is j + k
-                // row j + KB enters the window: its input, from chunk c or c + 1 of the ring
-                const c2<T> vin = Vb[((c + (jj + KB) / PCH) % ROT_VRING) * PCH + (jj + KB) % PCH];
-                if (k == KB) w = vin;
-                c2<T> lcur = (k >= 1 && k <= KB) ? Lc[jj * KB + k - 1] : mk<T>(0, 0);
-                const int pj = Pc[jj] - j;
-                const int l0 = j & 31, lp = (j + pj) & 31;
-                c2<T> zj = shfl2<T>(w, lp), w0 = shfl2<T>(w, l0);
-                if (lane == lp && pj != 0) w = w0;   // recorded interchange of rows j and j + pj
-                if (k >= 1 && k <= KB && j + k < n) {
-                    w.x -= lcur.x * zj.x - lcur.y * zj.y;
-                    w.y -= lcur.x * zj.y + lcur.y * zj.x;
+            for (int jj = 0; jj < W; jj++) {
+                const c2<T> lf = f[jj];
+                const int q = (pq[jj / 4] >> (8 * (jj % 4))) & 255;   // the pivot row's lane
+                const c2<T> zj = mk<T>(__shfl_sync(0xffffffffu, w.x, q, W), __shfl_sync(0xffffffffu, w.y, q, W));
+                const c2<T> w0 = mk<T>(__shfl_sync(0xffffffffu, w.x, jj, W), __shfl_sync(0xffffffffu, w.y, jj, W));
+                if (l == q) w = w0;   // recorded interchange
+                sub_prod<T>(w, lf, zj);
+                if (l == jj) {
+                    out = zj;
+                    w = wn;
                 }
-                if (lane == l0) zo[j] = zj;
+                f[jj] = Fn[jj * W];
             }
-            __syncwarp();   // buffers (c & 1) and ring slot c are refilled by later copies
+            const int row = c * W + l;
+            if (ok && row < n) zo[row] = sizeof(T) == 8 ? cm_pin<T>(out, di) : out;
+            wn = input(nxt, (c + 2) * W + l);
+#pragma unroll
+            for (int e = 0; e < W / 4; e++) pq[e] = pn[e];
         }
-        __syncwarp();   // the forward results are visible to the warp's copies below
-        // backward group q (chunk c = nc - 1 - q): factor chunk c and forward-result chunk c
-        auto issue_bwd = [&](int c, int bb) {
-            int i0 = c * PCH, rows = min(PCH, n - i0);
-            warp_copy16(Ub + bb * PCH * (WU + 1), Uk + (int64_t)i0 * (WU + 1), rows * (WU + 1) * (int)sizeof(c2<T>),
-                        lane);
-            warp_copy16(Db + bb * PCH, Dk + i0, rows * (int)sizeof(c2<T>), lane);
-            copy_vec(zo, c);
-            cp_async_commit();
+        // backward; a lane reads the forward results that it stored itself
+        auto fwd = [&](int c) {
+            const int row = c * W + l;
+            return ok && c >= 0 && row < n ? zo[row] : mk<T>(0, 0);
         };
-        issue_bwd(nc - 1, 0);
-        // backward: lane l holds row i - m, m = (i - l) mod 32; rows i - 1 .. i - WU accumulate
-        c2<T> acc = mk<T>(0, 0), x = mk<T>(0, 0);
-        for (int q = 0; q < nc; q++) {
-            const int c = nc - 1 - q;
-            if (c > 0) {
-                issue_bwd(c - 1, (q + 1) & 1);
-                cp_async_wait1();
-            } else {
-                cp_async_wait0();
-            }
-            __syncwarp();
-            const c2<T>* Uc = Ub + (q & 1) * PCH * (WU + 1);
-            const c2<T>* Dc = Db + (q & 1) * PCH;
-            const c2<T>* Zc = Vb + (c % ROT_VRING) * PCH;
-            const int i0 = c * PCH, rows = min(PCH, n - i0);
 #pragma unroll
-            for (int iq = 0; iq < PCH; iq++) {
-                const int ii = rows - 1 - iq;
-                if (ii < 0) break;
-                const int i = i0 + ii;
-                const int m = (i - lane) & 31;
-                c2<T> ucur = (m >= 1 && m <= WU && i - m >= 0) ? Uc[ii * (WU + 1) + m] : mk<T>(0, 0);
-                const c2<T> zi = Zc[ii], di = Dc[ii];
-                if (m == 0) x = cm<T>(mk<T>(zi.x - acc.x, zi.y - acc.y), di);
-                c2<T> xi = shfl2<T>(x, i & 31);
-                if (m >= 1 && m <= WU) {
-                    acc.x += ucur.x * xi.x - ucur.y * xi.y;
-                    acc.y += ucur.x * xi.y + ucur.y * xi.x;
+        for (int jj = 0; jj < W; jj++) f[jj] = Bp[(int64_t)(nc - 1) * (W * W) + jj * W];
+        for (int c = 1; c < AHEAD; c++) fetch(Bp, nc - 1 - c);
+        c2<T> acc = mk<T>(0, 0), zc = fwd(nc - 1), zn = fwd(nc - 2);
+        if (sizeof(T) == 8) acc = zc;
+        for (int c = nc - 1; c >= 0; c--) {
+            const c2<T> nxt = fwd(c - 2);
+            fetch(Bp, c - AHEAD);
+            const c2<T>* Bn = Bp + (int64_t)max(c - 1, 0) * (W * W);
+#pragma unroll
+            for (int jj = W - 1; jj >= 0; jj--) {
+                const c2<T> u = f[jj];
+                // in the row's lane u = 1 / U[i][i]
+                const c2<T> x = sizeof(T) == 8 ? acc : cm<T>(mk<T>(zc.x - acc.x, zc.y - acc.y), u);
+                const c2<T> xi = mk<T>(__shfl_sync(0xffffffffu, x.x, jj, W), __shfl_sync(0xffffffffu, x.y, jj, W));
+                add_back<T>(acc, u, xi);
+                if (l == jj) {
+                    out = xi;
+                    acc = sizeof(T) == 8 ? zn : mk<T>(0, 0);
+                    zc = zn;
                 }
-                if (m == 0) {
-                    zo[i] = xi;
-                    acc = mk<T>(0, 0);   // the lane's next row is i - 32
-                }
+                f[jj] = Bn[jj * W];
             }
-            __syncwarp();
+            const int row = c * W + l;
+            if (ok && row < n) zo[row] = out;
+            zn = nxt;
         }
     }
-    if (part_nrm) block_reduce_store(make_double2(0, 0), nsum, nullptr, part_nrm, blockIdx.x);
-}
-
-template <class T>
-size_t precond_rot_smem()
-{
-    return (size_t)prec_rot_warps<T>() * prec_rot_warp_bytes<T, 13>();
-}
-
-template <class T>
-cudaError_t precond_rot_prepare()
-{
-    return cudaFuncSetAttribute(k_precond_rot<T, 13>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)precond_rot_smem<T>());
+    if (part_nrm) {
+        // summed in the order of the other schedules: 32 lanes of a channel, then the block's channels
+        __shared__ double wsum[CPB];
+        double ns = W == 16 ? n0 + n1 : n0;
+#pragma unroll
+        for (int off = W / 2; off > 0; off >>= 1) ns += __shfl_down_sync(0xffffffffu, ns, off, W);
+        if (l == 0) wsum[slot] = ns;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0;
+            for (int w = 0; w < CPB; w++) t += wsum[w];
+            part_nrm[blockIdx.x] = t;
+        }
+    }
 }
 
 template <class T>
 int precond_rot_blocks(int nch)
 {
-    return (nch + prec_rot_warps<T>() - 1) / prec_rot_warps<T>();
+    return (nch + rot_cpb<T>() - 1) / rot_cpb<T>();
 }
 
 template <class T>
-void launch_precond_rot_t(cudaStream_t st, const OpView& A, const void* U, const void* L, const void* Dinv, int mode,
-                          const KState* ks, const void* r, const void* v, void* io, void* z, double* pn)
+void launch_precond_rot_t(cudaStream_t st, const OpView& A, int lanes, const void* F, const void* Bk,
+                          const void* Dinv, const uint4* piv,
+                          int mode, const KState* ks, const void* r, const void* v, void* io, void* z, double* pn)
 {
-    k_precond_rot<T, 13><<<precond_rot_blocks<T>(A.nch), 32 * prec_rot_warps<T>(), precond_rot_smem<T>(), st>>>(
-        A, (const c2<T>*)U, (const c2<T>*)L, (const c2<T>*)Dinv, mode, ks, (const c2<T>*)r, (const c2<T>*)v,
-        (c2<T>*)io, (c2<T>*)z, pn);
+    auto kernel = lanes == 16 ? k_precond_rot<T, 16> : k_precond_rot<T, 32>;
+    kernel<<<precond_rot_blocks<T>(A.nch), rot_cpb<T>() * lanes, 0, st>>>(
+        A, (const c2<T>*)F, (const c2<T>*)Bk, (const c2<T>*)Dinv, piv, mode, ks, (const c2<T>*)r, (const c2<T>*)v, (c2<T>*)io, (c2<T>*)z, pn);
 }
-template cudaError_t precond_rot_prepare<double>();
-template cudaError_t precond_rot_prepare<float>();
 template int precond_rot_blocks<double>(int);
 template int precond_rot_blocks<float>(int);
-template void launch_precond_rot_t<double>(cudaStream_t, const OpView&, const void*, const void*, const void*, int,
+template void launch_precond_rot_t<double>(cudaStream_t, const OpView&, int, const void*, const void*, const void*, const uint4*, int,
                                            const KState*, const void*, const void*, void*, void*, double*);
-template void launch_precond_rot_t<float>(cudaStream_t, const OpView&, const void*, const void*, const void*, int,
+template void launch_precond_rot_t<float>(cudaStream_t, const OpView&, int, const void*, const void*, const void*, const uint4*, int,
                                           const KState*, const void*, const void*, void*, void*, double*);
 
 template <class T>

@@ -22,6 +22,7 @@ struct Krylov {
     KState* ks = nullptr;
     const void *S = nullptr, *H = nullptr, *W = nullptr, *U = nullptr, *L = nullptr;
     const void *Urow = nullptr, *Dinv = nullptr;   // lane-per-channel preconditioner data
+    const void *rotF = nullptr, *rotB = nullptr;   // rotated-lane preconditioner's factor tables
 };
 
 struct GraphDriver;   // graph.cu
@@ -62,6 +63,8 @@ struct dirac_op {
     int prec_sched32 = 0, prec_sched64 = 1;
     bool prec_sm_ok = false;     // the staged kernel fits this radial size
     bool prec_rot_ok = false;    // the rotated-lane kernel is set up (band width 13)
+    int rot_lanes = 16;          // its lanes per channel
+    uint4* rot_piv = nullptr;    // its pivot lanes
     float prec_ms32[4] = {0, 0, 0, 0}, prec_ms64[4] = {0, 0, 0, 0};
     int config_gen = 0;          // bumped when a launch choice changes (captured graphs are rebuilt)
     int *wks = nullptr, *wfirst = nullptr, *wcnt = nullptr;
