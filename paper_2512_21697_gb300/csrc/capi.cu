@@ -129,6 +129,7 @@ void collect_phases(dirac_op* op)
 int apply_parts(const dirac_op* op, const Krylov& K)
 {
     if (op->use_ang && (K.prec == 0 || op->fact32 != 2)) return rad_parts(K.prec, op->ov.n1, op->nrad_lanes);
+    if (K.prec == 0 && op->split64) return apply_split_parts(op->ov.nch, op->ov.n1);
     if (K.prec == 1 && op->fact32 == 1) return grid_for(op->ov.n1, FTR) * op->nfsub;
     if (K.prec == 1 && op->fact32 == 2) return grid_for(op->ov.n1, FTR) * op->ov.nch;
     return (K.prec == 1 && op->part_own) ? op->nparts_own : op->nparts_apply;
@@ -143,7 +144,10 @@ void k_apply_launch(dirac_op* op, const Krylov& K, int sign, const void* x, void
         op->launches++;
         launch_ang64(op->st, op->ov, op->ang4, op->ang_c64, op->rad_lanes, op->nrad_lanes, op->Ed, (const double*)K.S,
                      (const double*)K.H, sign, x, op->ang_S, y, bsub, dv, pdot, pnrm, skip);
-    } else if (K.prec == 0)
+    } else if (K.prec == 0 && op->split64)
+        launch_apply_split(op->st, op->ov, (const double*)K.S, (const double*)K.H, sign, x, (const double*)K.W, y, bsub,
+                           dv, pdot, pnrm, skip);
+    else if (K.prec == 0)
         launch_apply_t<double>(grid, op->st, op->ov, (const double*)K.S, (const double*)K.H, sign, x,
                                (const double*)K.W, y, bsub, dv, pdot, pnrm, skip);
     else if (op->use_ang && op->fact32 != 2) {
@@ -1374,11 +1378,15 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
         }
     }
     op->nparts_apply = grid_for(n1, 128) * B.nch;
+    // Two FP64 applies with their reductions (row kernel / split): 1.02 .. 1.30 up to 31920 blocks of the
+    // split kernel, 0.97 .. 1.01 at 63840 .. 204624 -- the row kernel's blocks fill the chip there, and the
+    // final sum takes 0.8 us per 1024 partials.
+    op->split64 = apply_split_parts(B.nch, n1) <= 32768;
     op->nparts_own = grid_for(n1, apply_own_tile()) * B.nch;
     op->nparts_vec = grid_for(op->n, 256);
     op->nparts_prec = grid_for(B.nch, 4);                     // ||s||^2 partials, warp-per-channel kernel
     op->nparts_prec32 = op->prec_warps ? op->prec_warps : grid_for(B.nch, 4);   // lane-per-channel kernel
-    int np = std::max({op->nparts_apply, op->nparts_own, op->nparts_vec, op->nparts_prec, op->nparts_prec32,
+    int np = std::max({op->nparts_apply, op->split64 ? apply_split_parts(B.nch, n1) : 0, op->nparts_own, op->nparts_vec, op->nparts_prec, op->nparts_prec32,
                        grid_for(n1, FTR) * B.nch, op->ang ? rad_parts(0, n1, op->nrad_lanes) : 0,
                        op->ang ? rad_parts(1, n1, op->nrad_lanes) : 0,
                        precond_sm_blocks<double>(B.nch), precond_sm_blocks<float>(B.nch),

@@ -137,6 +137,12 @@ template <class T>
 void launch_precond_sm_t(cudaStream_t st, const OpView& A, const void* U, const void* L, const void* Dinv, int mode,
                          const KState* ks, const void* r, const void* v, void* io, void* z, double* pn);
 
+// FP64 apply split over the partners (small systems); apply_split_parts partials
+int apply_split_parts(int nch, int n1);
+void launch_apply_split(cudaStream_t st, const OpView& A, const double* S, const double* H, int sign, const void* x,
+                        const double* W, void* y, const void* bsub, const void* dv, double2* pdot, double* pnrm,
+                        const KState* skip);
+
 // rotated-lane preconditioner (band width 13), 16 or 32 lanes per channel; F, Bk, piv: its factor tables
 // [kappa slot][row, padded to a multiple of lanes][lane] and pivot lanes [kappa slot][row]
 template <class T> int precond_rot_blocks(int nch);

@@ -139,6 +139,117 @@ __global__ void __launch_bounds__(128) k_apply(OpView A, const T* __restrict__ S
     }
 }
 
+// The same product in FP64 for systems too small to fill the chip with k_apply's blocks: SR rows of a
+// channel per block, the partners of a row (and the diagonal block's 13 positions) dealt to SG threads and
+// their sums added in a fixed order.  What bounds such a system is the FP64 unit of the few SMs in use (a
+// warp's operation takes it 16 cycles), so the work has to reach all of them.  Per apply, row kernel -> this:
+// 57 -> 14 us at 16 channels and 61 slots, 122 -> 33 us at 84 and 61, 111 -> 80 us at 40 and 601, 846 -> 734
+// us at 220 and 601.
+constexpr int SR = 8, SG = 16;
+
+template <int BD>
+__global__ void __launch_bounds__(SR * SG) k_apply_split(OpView A, const double* __restrict__ S,
+                                                         const double* __restrict__ H, int sign,
+                                                         const double2* __restrict__ x, const double* __restrict__ W,
+                                                         double2* __restrict__ y, const double2* __restrict__ bsub,
+                                                         const double2* __restrict__ dv, double2* part_dot,
+                                                         double* part_nrm, const KState* skip)
+{
+    if (skip && skip->done) return;   // uniform over the grid: the solve already finished
+    const int bd = BD > 0 ? BD : A.bd, half = (bd - 1) / 2, n1 = A.n1;
+    const int ch = blockIdx.x, row = threadIdx.x % SR, g = threadIdx.x / SR, r = blockIdx.y * SR + row;
+    double2 y0 = make_double2(0, 0), y1 = y0;
+    if (r < n1) {
+        const double2* xa = x + (int64_t)ch * 2 * n1;
+        const int64_t k0 = ((int64_t)A.ch_kslot[ch] * n1 + r) * bd * 4;
+        const double st = sign * A.tau;
+        for (int d = g; d < bd; d += SG) {
+            const int rr = r + d - half;
+            if (rr < 0 || rr >= n1) continue;
+            const double2 x0 = xa[2 * rr], x1 = xa[2 * rr + 1];
+            const double *s = S + k0 + d * 4, *hp = H + k0 + d * 4;
+            const double h[4] = {st * hp[0], st * hp[1], st * hp[2], st * hp[3]};
+            y0.x = fma(s[0], x0.x, fma(s[1], x1.x, fma(-h[0], x0.y, fma(-h[1], x1.y, y0.x))));
+            y0.y = fma(s[0], x0.y, fma(s[1], x1.y, fma(h[0], x0.x, fma(h[1], x1.x, y0.y))));
+            y1.x = fma(s[2], x0.x, fma(s[3], x1.x, fma(-h[2], x0.y, fma(-h[3], x1.y, y1.x))));
+            y1.y = fma(s[2], x0.y, fma(s[3], x1.y, fma(h[2], x0.x, fma(h[3], x1.x, y1.y))));
+        }
+        for (int e = A.adj_start[ch] + g; e < A.adj_start[ch + 1]; e += SG) {
+            const double2* xb = x + (int64_t)A.adj_nbr[e] * 2 * n1;
+            const double* Wp = W + (int64_t)A.adj_pair[e] * n1 * bd * 4;
+            const bool tr = A.adj_tr[e];   // -sign W x_b, or sign W^T x_b
+            const long long flip = (tr ? sign : -sign) < 0 ? 1LL << 63 : 0;
+            auto signed_ = [&](double v) { return __longlong_as_double(__double_as_longlong(v) ^ flip); };
+#pragma unroll
+            for (int d = 0; d < bd; d++) {
+                const int rr = r + d - half;
+                if (rr < 0 || rr >= n1) continue;
+                const double2* w = reinterpret_cast<const double2*>(
+                    Wp + (int64_t)(tr ? rr * bd + 2 * half - d : r * bd + d) * 4);
+                const double2 wa = w[0], wb = w[1];
+                const double w01 = tr ? wb.x : wa.y, w10 = tr ? wa.y : wb.x;
+                double2 x0 = xb[2 * rr], x1 = xb[2 * rr + 1];
+                x0.x = signed_(x0.x); x0.y = signed_(x0.y);
+                x1.x = signed_(x1.x); x1.y = signed_(x1.y);
+                y0.x = fma(wa.x, x0.x, y0.x); y0.y = fma(wa.x, x0.y, y0.y);
+                y1.x = fma(w10, x0.x, y1.x); y1.y = fma(w10, x0.y, y1.y);
+                y0.x = fma(w01, x1.x, y0.x); y0.y = fma(w01, x1.y, y0.y);
+                y1.x = fma(wb.y, x1.x, y1.x); y1.y = fma(wb.y, x1.y, y1.y);
+            }
+        }
+    }
+    // the groups' sums: entry (row, component) by four threads of four groups each, then by one
+    static_assert(SR * 4 == 32 && SG == 16, "the sums below are laid out for 32 entries of 16 groups");
+    __shared__ double red[SG][33];
+    red[g][row * 4] = y0.x; red[g][row * 4 + 1] = y0.y; red[g][row * 4 + 2] = y1.x; red[g][row * 4 + 3] = y1.y;
+    __syncthreads();
+    const int v = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const double part = (red[4 * q][v] + red[4 * q + 1][v]) + (red[4 * q + 2][v] + red[4 * q + 3][v]);
+    __syncthreads();
+    red[q][v] = part;
+    __syncthreads();
+    if (q) return;
+    const int rv = blockIdx.y * SR + v / 4;
+    const bool act = rv < n1;
+    double yv = (red[0][v] + red[1][v]) + (red[2][v] + red[3][v]), dx = 0, dy = 0, ns = 0;
+    if (act) {
+        const int64_t o = (int64_t)ch * 2 * n1 + 2 * rv + (v % 4) / 2;   // complex entry
+        const int c = v & 1;
+        if (bsub) yv = reinterpret_cast<const double*>(bsub)[2 * o + c] - yv;
+        reinterpret_cast<double*>(y)[2 * o + c] = yv;
+        if (dv) {
+            const double2 a = dv[o];
+            dx = (c ? a.y : a.x) * yv;
+            dy = (c ? a.x : -a.y) * yv;
+        }
+        ns = yv * yv;
+    }
+    const int64_t slot = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
+    for (int off = 16; off > 0; off >>= 1) {
+        if (part_dot) {
+            dx += __shfl_down_sync(0xffffffffu, dx, off);
+            dy += __shfl_down_sync(0xffffffffu, dy, off);
+        }
+        if (part_nrm) ns += __shfl_down_sync(0xffffffffu, ns, off);
+    }
+    if (v == 0) {
+        if (part_dot) part_dot[slot] = make_double2(dx, dy);
+        if (part_nrm) part_nrm[slot] = ns;
+    }
+}
+
+int apply_split_parts(int nch, int n1) { return nch * ((n1 + SR - 1) / SR); }
+
+void launch_apply_split(cudaStream_t st, const OpView& A, const double* S, const double* H, int sign, const void* x,
+                        const double* W, void* y, const void* bsub, const void* dv, double2* pdot, double* pnrm,
+                        const KState* skip)
+{
+    auto kernel = A.bd == 13 ? k_apply_split<13> : k_apply_split<0>;
+    kernel<<<dim3(A.nch, (A.n1 + SR - 1) / SR), SR * SG, 0, st>>>(A, S, H, sign, (const double2*)x, W, (double2*)y,
+                                                                  (const double2*)bsub, (const double2*)dv, pdot, pnrm,
+                                                                  skip);
+}
+
 template <class T>
 void launch_apply_t(dim3 grid, cudaStream_t st, const OpView& A, const T* S, const T* H, int sign, const void* x,
                     const T* W, void* y, const void* bsub, const void* dv, double2* pdot, double* pnrm,

@@ -57,6 +57,7 @@ struct dirac_op {
     // block partials written by each kind of launch (the reductions must read exactly these):
     // nparts_apply: 128-row tiles (FP64 apply, observables); nparts_own: the owner/gather passes
     int nparts_apply = 0, nparts_own = 0, nparts_vec = 0, nparts_prec = 0, nparts_prec32 = 0;
+    bool split64 = false;        // the FP64 apply is split over the partners (k_apply_split)
     int prec_warps = 0;          // same-kappa channel groups (lane-per-channel preconditioner)
     // preconditioner schedules, picked by timing at setup: 0 one lane per channel (complex64 only),
     // 1 one warp per channel, 2 one warp per channel with shared-memory staging

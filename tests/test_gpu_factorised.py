@@ -100,6 +100,31 @@ def test_fp64_products_match_oracle_rows(oracle_mod, kmax, N, lmax, precision):
         assert np.abs(yn[rows] - ref).max() <= 64 * (2 * m + 8) * U32 * 4 * np.abs(yn).max()
 
 
+# stored FP64 products: the kernel split over the partners (radial slots at the edges of its 8-row blocks, the
+# largest grid) and the row kernel above
+@pytest.mark.parametrize("kmax,N,lmax", [(3, 40, 1), (4, 47, 2), (4, 48, 2), (30, 135, 1), (30, 143, 1)])
+def test_stored_fp64_product_matches_oracle_rows(oracle_mod, kmax, N, lmax):
+    import torch
+    cfg, bas, orc, perm, inv, rows, psi = _case(oracle_mod, kmax, N, lmax, 64)
+    t = 0.57 * cfg["n_cycles"] * 2 * math.pi / cfg["omega"]
+    ch, idx = rows // orc.nb, rows % orc.nb
+    op = B.Operator(bas, cfg, tol=1e-10, precision=1, tol_inner=1e-5, max_outer=20)
+    xd = torch.from_numpy(psi[inv]).cuda()
+    y = torch.empty_like(xd)
+    ys = {}
+    for sign in (+1, -1):
+        op.apply(sign, t, xd, y)
+        yn = ys[sign] = y.cpu().numpy()[perm]
+        assert np.abs(yn[rows] - orc.apply_rows(t, sign, psi, ch, idx)).max() <= 1e-12 * np.abs(yn).max()
+        assert np.all(yn[~orc.active_mask()] == 0)
+    # the residual's epilogues: r = b - A_+ x and ||b||
+    r = torch.empty_like(xd)
+    bn = op.residual(t, xd, xd, r)
+    scale = max(np.abs(ys[1]).max(), np.abs(ys[-1]).max())
+    assert np.abs(r.cpu().numpy()[perm] - (ys[-1] - ys[1])).max() <= 1e-12 * scale
+    assert abs(bn - np.linalg.norm(ys[-1])) <= 1e-12 * bn
+
+
 @pytest.mark.parametrize("precision,tol", [(0, 1e-10), (1, 1e-10), (2, 1e-10), (2, 1e-12)])
 def test_drivers_agree_and_modes_switch(precision, tol):
     # host loop, overlapped assembly, captured driver: the same arithmetic, bit for bit, with single
