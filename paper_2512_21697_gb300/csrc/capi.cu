@@ -343,6 +343,15 @@ void residual_accurate(dirac_op* op, const void* psi)
     finish(op, K.ks, 1, op->nparts_apply, nullptr, op->part_n, op->opts.max_iter);
 }
 
+// Whether a schedule runs the rotated-lane kernel: schedule 3 (order 7), and, at the other spline orders,
+// schedule 1, which is their only one: the same operations in the same order.  At 420 channels and 601
+// slots of order 8, complex64 101 us against the shifting-window kernel's 505, complex128 492 against 1320;
+// at 40 channels and 61 slots of order 5, 17 against 50 and 54 against 127.
+static bool rot_runs(const dirac_op* op, int sched)
+{
+    return op->rot_piv && (sched == 3 ? op->prec_rot_ok : op->ov.bd != 13);
+}
+
 void k_precond_launch(dirac_op* op, const Krylov& K, int mode, const KState* ks, const void* r,
                              const void* v, void* io, void* z, double* pn)
 {
@@ -356,7 +365,7 @@ void k_precond_launch(dirac_op* op, const Krylov& K, int mode, const KState* ks,
                                           op->wcnt, mode, ks, r, v, io, z, pn);
         else if (op->prec_sched32 == 2 && op->prec_sm_ok)
             launch_precond_sm_t<float>(op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z, pn);
-        else if (op->prec_sched32 == 3 && op->prec_rot_ok)
+        else if (rot_runs(op, op->prec_sched32))
             launch_precond_rot_t<float>(op->st, op->ov, op->rot_lanes, K.rotF, K.rotB, K.Dinv, op->rot_piv, mode, ks, r, v, io, z, pn);
         else
             launch_precond_t<float>(grid_for(op->ov.nch, 4), op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z,
@@ -364,7 +373,7 @@ void k_precond_launch(dirac_op* op, const Krylov& K, int mode, const KState* ks,
     } else {
         if (op->prec_sched64 == 2 && op->prec_sm_ok)
             launch_precond_sm_t<double>(op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z, pn);
-        else if (op->prec_sched64 == 3 && op->prec_rot_ok)
+        else if (rot_runs(op, op->prec_sched64))
             launch_precond_rot_t<double>(op->st, op->ov, op->rot_lanes, K.rotF, K.rotB, K.Dinv, op->rot_piv, mode, ks, r, v, io, z, pn);
         else
             launch_precond_t<double>(grid_for(op->ov.nch, 4), op->st, op->ov, K.U, K.L, K.Dinv, mode, ks, r, v, io, z,
@@ -377,11 +386,11 @@ int prec_parts(const dirac_op* op, const Krylov& K)
     if (K.prec == 1) {
         if (op->prec_sched32 == 0 && op->prec_warps) return op->prec_warps;
         if (op->prec_sched32 == 2 && op->prec_sm_ok) return precond_sm_blocks<float>(op->ov.nch);
-        if (op->prec_sched32 == 3 && op->prec_rot_ok) return precond_rot_blocks<float>(op->ov.nch);
+        if (rot_runs(op, op->prec_sched32)) return precond_rot_blocks<float>(op->ov.nch);
         return grid_for(op->ov.nch, 4);
     }
     if (op->prec_sched64 == 2 && op->prec_sm_ok) return precond_sm_blocks<double>(op->ov.nch);
-    if (op->prec_sched64 == 3 && op->prec_rot_ok) return precond_rot_blocks<double>(op->ov.nch);
+    if (rot_runs(op, op->prec_sched64)) return precond_rot_blocks<double>(op->ov.nch);
     return grid_for(op->ov.nch, 4);
 }
 
@@ -1098,8 +1107,9 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     // zero elsewhere.  16 lanes hold the backward window if U's superdiagonals from 16 on are zero.
     std::vector<double2> hRF, hRB;
     double2 *dRF = nullptr, *dRB = nullptr;
-    if (bd == 13) {
-        int W = 16;
+    const bool rot = wu < 32;
+    if (rot) {
+        int W = kb < 16 ? 16 : 32;
         for (size_t e = 0; e < hU.size(); e++)
             if (e % (wu + 1) >= 16 && (hU[e].x != 0 || hU[e].y != 0)) W = 32;
         const size_t np = (size_t)(ns + W - 1) / W * W;
@@ -1297,7 +1307,7 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
         TRY(upload(op, &fdUr, fUr));
         TRY(upload(op, &fdDi, fDi));
         op->k32.Urow = fdUr; op->k32.Dinv = fdDi;
-        if (bd == 13) {
+        if (rot) {
             float2 *fRF, *fRB;
             TRY(upload(op, &fRF, tof(hRF)));
             TRY(upload(op, &fRB, tof(hRB)));

@@ -802,8 +802,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 template <class T, int W>
 __global__ void __launch_bounds__(rot_cpb<T>() * W) k_precond_rot(
     OpView A, const c2<T>* __restrict__ F, const c2<T>* __restrict__ Bk, const c2<T>* __restrict__ Dinv,
-    const uint4* __restrict__ piv, int mode, const KState* st, const c2<T>* __restrict__ r, const c2<T>* __restrict__ v, c2<T>* __restrict__ io,
-    c2<T>* __restrict__ z, double* part_nrm)
+    const uint4* __restrict__ piv, int mode, const KState* st, const c2<T>* __restrict__ r,
+    const c2<T>* __restrict__ v, c2<T>* __restrict__ io, c2<T>* __restrict__ z, double* part_nrm)
 {
     constexpr int CPB = rot_cpb<T>(), AHEAD = 4;
     const int l = threadIdx.x % W, slot = threadIdx.x / W, pos = blockIdx.x * CPB + slot;
