@@ -35,7 +35,7 @@ constexpr int GN_IN = 32, GN_H = 256, GN_OUT = 4;
 constexpr int64_t GO_W1 = 0, GO_B1 = GO_W1 + GN_IN * GN_H, GO_W2 = GO_B1 + GN_H, GO_B2 = GO_W2 + GN_H * GN_H,
                   GO_W3 = GO_B2 + GN_H, GO_B3 = GO_W3 + GN_H * GN_H, GO_W4 = GO_B3 + GN_H,
                   GO_B4 = GO_W4 + GN_H * GN_OUT, GN_PARAMS = GO_B4 + GN_OUT;
-constexpr int GCHUNK = 1024;   // samples per partial of a gradient reduction
+constexpr int GCHUNK = 1024;   // samples per partial of the loss
 
 }  // namespace dg
 
@@ -49,8 +49,8 @@ struct dirac_guess {
     int* err = nullptr;             // error word of the tcgen05 forward's bounded waits
     float *m = nullptr, *v = nullptr, *g = nullptr;
     float *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *out = nullptr;   // training activations
-    float *d1 = nullptr, *d2 = nullptr, *dout = nullptr;                 // back-propagated errors
-    float* part = nullptr;          // split-sample partial gradients
+    float *d1 = nullptr, *d2 = nullptr, *d3 = nullptr, *dout = nullptr;  // back-propagated errors
+    float* part = nullptr;          // split-sample partial gradients, each laid out as the parameters
     double* lpart = nullptr;        // loss partials
     double* hloss = nullptr;        // pinned host loss
 };
@@ -191,37 +191,64 @@ __global__ void k_guess_apply(int64_t npos, const double2* __restrict__ p0, cons
 // FP32 tiled GEMM with epilogues (training path and the reference forward)
 //   C[i][j] = epi( sum_k A[i][k] B'[k][j] ),  B' = B (K x N, row-major) or B^T (B is N x K)
 //   epi: 0 = + bias, 1 = tanh(. + bias), 2 = . * (1 - G[i][j]^2) (back-propagation through tanh)
-// 64 x 64 tile per block of 256 threads, 4 x 4 outputs per thread, K in chunks of 16.
+// 64 x 64 tile per block of 256 threads, 4 x 4 outputs per thread, K in chunks of 32: a block of two warps a
+// scheduler has little to hide a load behind, so the next chunk's entries are on their way in registers
+// while a chunk is used.  The sums run over k in order.  42 -> 26 us at 4096 x 256 x 256 against chunks of 16
+// loaded and used in turn.
 // ------------------------------------------------------------------------------------------
+constexpr int GK = 32, GS = 64 + 4;   // chunk length, row stride of a staged chunk (16-byte rows)
+
+// acc += (the thread's four columns of a) (its four of b) over the rows of a staged chunk
+__device__ __forceinline__ void chunk_fma(float (&acc)[4][4], const float (*As)[GS], const float (*Bs)[GS], int tx, int ty)
+{
+#pragma unroll
+    for (int kk = 0; kk < GK; kk++) {
+        const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
+        const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
+        const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
+    }
+}
+
 template <bool TB, int EPI>
 __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* __restrict__ A,
                                               const float* __restrict__ B, const float* __restrict__ bias,
                                               const float* __restrict__ G, float* __restrict__ C)
 {
-    __shared__ float As[16][64 + 4];
-    __shared__ float Bs[16][64 + 4];
-    int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-            int ii = e / 16, kk = e % 16;
-            int gi = i0 + ii, gk = k0 + kk;
-            As[kk][ii] = (gi < M && gk < K) ? A[(int64_t)gi * K + gk] : 0.f;
-            int jj = e % 64, kb = e / 64;
-            int gj = j0 + jj, gkb = k0 + kb;
-            float bv = 0.f;
-            if (gj < N && gkb < K) bv = TB ? B[(int64_t)gj * K + gkb] : B[(int64_t)gkb * N + gj];
-            Bs[kb][jj] = bv;
-        }
-        __syncthreads();
+    __shared__ __align__(16) float As[2][GK][GS], Bs[2][GK][GS];
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4, i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
+    constexpr int NL = 64 * GK / 256;
+    float ra[NL], rb[NL];
+    auto fetch = [&](int k0) {
 #pragma unroll
-        for (int kk = 0; kk < 16; kk++) {
-            float a[4], b[4];
-            for (int q = 0; q < 4; q++) { a[q] = As[kk][ty * 4 + q]; b[q] = Bs[kk][tx * 4 + q]; }
-            for (int p = 0; p < 4; p++)
-                for (int q = 0; q < 4; q++) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
+        for (int u = 0; u < NL; u++) {
+            const int e = t + 256 * u, gi = i0 + e / GK, gk = k0 + e % GK;
+            ra[u] = gi < M && gk < K ? A[(int64_t)gi * K + gk] : 0.f;
+            const int gj = j0 + (TB ? e / GK : e % 64), gkb = k0 + (TB ? e % GK : e / 64);
+            rb[u] = gj < N && gkb < K ? (TB ? B[(int64_t)gj * K + gkb] : B[(int64_t)gkb * N + gj]) : 0.f;
         }
+    };
+    auto stash = [&](int b) {
+#pragma unroll
+        for (int u = 0; u < NL; u++) {
+            const int e = t + 256 * u;
+            As[b][e % GK][e / GK] = ra[u];
+            if (TB) Bs[b][e % GK][e / GK] = rb[u];
+            else Bs[b][e / 64][e % 64] = rb[u];
+        }
+    };
+    float acc[4][4] = {};
+    fetch(0);
+    stash(0);
+    __syncthreads();
+    for (int k0 = 0, b = 0; k0 < K; k0 += GK, b ^= 1) {
+        const bool more = k0 + GK < K;
+        if (more) fetch(k0 + GK);
+        chunk_fma(acc, As[b], Bs[b], tx, ty);
+        if (more) stash(b ^ 1);   // last read before the previous barrier
         __syncthreads();
     }
     for (int p = 0; p < 4; p++) {
@@ -239,41 +266,66 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* 
     }
 }
 
-// partial weight gradient over one chunk of samples: P[chunk][k][j] = sum_{i in chunk} A[i][k] D[i][j]
-// (A: M x K, D: M x N); a 64 x 64 (k, j) tile per block
-__global__ void __launch_bounds__(256) k_gemm_tn_part(int M, int N, int K, const float* __restrict__ A,
-                                                      const float* __restrict__ D, float* __restrict__ P)
+// Partial gradients of every layer over one chunk of clen samples (blockIdx.y), laid out as the parameters,
+// P[chunk][parameter]: a weight gradient W[k][j] = sum_i A[i][k] D[i][j] in 64 x 64 tiles (blockIdx.x over the
+// layers' tiles), and with its first row of tiles the bias gradient b[j] = sum_i D[i][j].  The four layers
+// have 40 tiles, so the samples are split into up to 32 chunks to fill the chip: 50 us for 4096 samples,
+// against 665 us for one launch per layer over chunks of 1024 and 248 us for its column sums.
+struct GradJob {
+    const float *A, *D;
+    int K, N, first, jt;   // first block, tiles per row
+    int64_t wo, bo;        // parameter offsets of the weights and the biases
+};
+struct GradJobs { GradJob j[4]; };
+
+__global__ void __launch_bounds__(256) k_grad_part(int M, int clen, GradJobs jobs, float* __restrict__ P)
 {
-    __shared__ float As[16][64 + 4];
-    __shared__ float Ds[16][64 + 4];
-    int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    int k0 = blockIdx.y * 64, j0 = blockIdx.x * 64, chunk = blockIdx.z;
-    int ib = chunk * GCHUNK, ie = min(M, ib + GCHUNK);
-    float acc[4][4] = {};
-    for (int i1 = ib; i1 < ie; i1 += 16) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-            int ii = e / 64, cc = e % 64;
-            int gi = i1 + ii;
-            bool in = gi < ie;
-            As[ii][cc] = (in && k0 + cc < K) ? A[(int64_t)gi * K + k0 + cc] : 0.f;
-            Ds[ii][cc] = (in && j0 + cc < N) ? D[(int64_t)gi * N + j0 + cc] : 0.f;
-        }
-        __syncthreads();
+    __shared__ __align__(16) float As[2][GK][GS], Ds[2][GK][GS];
+    int q = 0;
+    while (q < 3 && (int)blockIdx.x >= jobs.j[q + 1].first) q++;
+    const GradJob& J = jobs.j[q];
+    const int tile = blockIdx.x - J.first, k0 = tile / J.jt * 64, j0 = tile % J.jt * 64, K = J.K, N = J.N;
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    const int ib = blockIdx.y * clen, ie = min(M, ib + clen);
+    constexpr int NL = 64 * GK / 256;
+    float ra[NL], rd[NL];
+    auto fetch = [&](int i1) {
 #pragma unroll
-        for (int ii = 0; ii < 16; ii++) {
-            float a[4], d[4];
-            for (int q = 0; q < 4; q++) { a[q] = As[ii][ty * 4 + q]; d[q] = Ds[ii][tx * 4 + q]; }
-            for (int p = 0; p < 4; p++)
-                for (int q = 0; q < 4; q++) acc[p][q] = fmaf(a[p], d[q], acc[p][q]);
+        for (int u = 0; u < NL; u++) {
+            const int e = t + 256 * u, gi = i1 + e / 64, cc = e % 64;
+            ra[u] = gi < ie && k0 + cc < K ? J.A[(int64_t)gi * K + k0 + cc] : 0.f;
+            rd[u] = gi < ie && j0 + cc < N ? J.D[(int64_t)gi * N + j0 + cc] : 0.f;
         }
+    };
+    auto stash = [&](int b) {
+#pragma unroll
+        for (int u = 0; u < NL; u++) {
+            const int e = t + 256 * u;
+            As[b][e / 64][e % 64] = ra[u];
+            Ds[b][e / 64][e % 64] = rd[u];
+        }
+    };
+    float acc[4][4] = {}, bsum = 0.f;
+    fetch(ib);
+    stash(0);
+    __syncthreads();
+    for (int i1 = ib, b = 0; i1 < ie; i1 += GK, b ^= 1) {
+        const bool more = i1 + GK < ie;
+        if (more) fetch(i1 + GK);
+        chunk_fma(acc, As[b], Ds[b], tx, ty);
+        if (k0 == 0 && t < 64)
+            for (int ii = 0; ii < GK; ii++) bsum += Ds[b][ii][t];
+        if (more) stash(b ^ 1);
         __syncthreads();
     }
+    float* Pc = P + (int64_t)blockIdx.y * GN_PARAMS;
+    if (k0 == 0 && t < 64 && j0 + t < N) Pc[J.bo + j0 + t] = bsum;
     for (int p = 0; p < 4; p++) {
-        int gk = k0 + ty * 4 + p;
+        const int gk = k0 + ty * 4 + p;
         if (gk >= K) continue;
-        for (int q = 0; q < 4; q++) {
-            int gj = j0 + tx * 4 + q;
-            if (gj < N) P[((int64_t)chunk * K + gk) * N + gj] = acc[p][q];
+        for (int c = 0; c < 4; c++) {
+            const int gj = j0 + tx * 4 + c;
+            if (gj < N) Pc[J.wo + (int64_t)gk * N + gj] = acc[p][c];
         }
     }
 }
@@ -286,17 +338,6 @@ __global__ void k_sum_chunks(int nchunk, int64_t KN, const float* __restrict__ P
     float s = 0.f;
     for (int c = 0; c < nchunk; c++) s += P[(int64_t)c * KN + e];
     G[e] = s;
-}
-
-// bias gradient: g[j] = sum_i D[i][j], chunked in the same fixed order
-__global__ void k_colsum_part(int M, int N, const float* __restrict__ D, float* __restrict__ P)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x, chunk = blockIdx.y;
-    if (j >= N) return;
-    int ib = chunk * GCHUNK, ie = min(M, ib + GCHUNK);
-    float s = 0.f;
-    for (int i = ib; i < ie; i++) s += D[(int64_t)i * N + j];
-    P[(int64_t)chunk * N + j] = s;
 }
 
 // dout = 2 (out - target) / B and per-chunk loss partials (double)
@@ -606,6 +647,9 @@ dirac_status gcheck(cudaError_t e, const char* what)
     } while (0)
 
 int nchunks(int B) { return (B + GCHUNK - 1) / GCHUNK; }
+// samples per partial of the parameter gradients: at most 32 partials, each of whole staged chunks
+constexpr int GPARTS = 32;
+int grad_chunk(int B) { return GK * ((B + GK * GPARTS - 1) / (GK * GPARTS)); }
 
 // forward through the FP32 kernels, keeping the activations (training and the reference path)
 void fwd32(dirac_guess* g, const float* X, int B, cudaStream_t st)
@@ -621,34 +665,26 @@ void fwd32(dirac_guess* g, const float* X, int B, cudaStream_t st)
 // loss and gradient into g->g (all parameters), loss partials into g->lpart
 void bwd32(dirac_guess* g, const float* X, const float* T, int B, cudaStream_t st)
 {
-    int nc = nchunks(B);
+    const int nc = nchunks(B), rows = (B + 63) / 64;
     dim3 b(256);
     const float* wr = g->wr;
-    float* P = g->part;
     k_loss_grad<<<nc, 256, 0, st>>>(B, g->out, T, g->dout, g->lpart);
-    // layer 4
-    k_gemm_tn_part<<<dim3(1, GN_H / 64, nc), b, 0, st>>>(B, GN_OUT, GN_H, g->a3, g->dout, P);
-    k_sum_chunks<<<(GN_H * GN_OUT + 255) / 256, 256, 0, st>>>(nc, GN_H * GN_OUT, P, g->g + GO_W4);
-    k_colsum_part<<<dim3(1, nc), 256, 0, st>>>(B, GN_OUT, g->dout, P);
-    k_sum_chunks<<<1, 256, 0, st>>>(nc, GN_OUT, P, g->g + GO_B4);
-    // d3 = (dout W4^T) (1 - a3^2) into d1 (scratch), then layer 3
-    k_gemm<true, 2><<<dim3(GN_H / 64, (B + 63) / 64), b, 0, st>>>(B, GN_H, GN_OUT, g->dout, wr + GO_W4, nullptr, g->a3, g->d1);
-    k_gemm_tn_part<<<dim3(GN_H / 64, GN_H / 64, nc), b, 0, st>>>(B, GN_H, GN_H, g->a2, g->d1, P);
-    k_sum_chunks<<<(GN_H * GN_H + 255) / 256, 256, 0, st>>>(nc, GN_H * GN_H, P, g->g + GO_W3);
-    k_colsum_part<<<dim3(1, nc), 256, 0, st>>>(B, GN_H, g->d1, P);
-    k_sum_chunks<<<1, 256, 0, st>>>(nc, GN_H, P, g->g + GO_B3);
-    // d2 = (d3 W3^T) (1 - a2^2), layer 2
-    k_gemm<true, 2><<<dim3(GN_H / 64, (B + 63) / 64), b, 0, st>>>(B, GN_H, GN_H, g->d1, wr + GO_W3, nullptr, g->a2, g->d2);
-    k_gemm_tn_part<<<dim3(GN_H / 64, GN_H / 64, nc), b, 0, st>>>(B, GN_H, GN_H, g->a1, g->d2, P);
-    k_sum_chunks<<<(GN_H * GN_H + 255) / 256, 256, 0, st>>>(nc, GN_H * GN_H, P, g->g + GO_W2);
-    k_colsum_part<<<dim3(1, nc), 256, 0, st>>>(B, GN_H, g->d2, P);
-    k_sum_chunks<<<1, 256, 0, st>>>(nc, GN_H, P, g->g + GO_B2);
-    // d1 = (d2 W2^T) (1 - a1^2), layer 1
-    k_gemm<true, 2><<<dim3(GN_H / 64, (B + 63) / 64), b, 0, st>>>(B, GN_H, GN_H, g->d2, wr + GO_W2, nullptr, g->a1, g->d1);
-    k_gemm_tn_part<<<dim3(GN_H / 64, 1, nc), b, 0, st>>>(B, GN_H, GN_IN, X, g->d1, P);
-    k_sum_chunks<<<(GN_IN * GN_H + 255) / 256, 256, 0, st>>>(nc, GN_IN * GN_H, P, g->g + GO_W1);
-    k_colsum_part<<<dim3(1, nc), 256, 0, st>>>(B, GN_H, g->d1, P);
-    k_sum_chunks<<<1, 256, 0, st>>>(nc, GN_H, P, g->g + GO_B1);
+    // d3 = (dout W4^T) (1 - a3^2), d2 = (d3 W3^T) (1 - a2^2), d1 = (d2 W2^T) (1 - a1^2)
+    k_gemm<true, 2><<<dim3(GN_H / 64, rows), b, 0, st>>>(B, GN_H, GN_OUT, g->dout, wr + GO_W4, nullptr, g->a3, g->d3);
+    k_gemm<true, 2><<<dim3(GN_H / 64, rows), b, 0, st>>>(B, GN_H, GN_H, g->d3, wr + GO_W3, nullptr, g->a2, g->d2);
+    k_gemm<true, 2><<<dim3(GN_H / 64, rows), b, 0, st>>>(B, GN_H, GN_H, g->d2, wr + GO_W2, nullptr, g->a1, g->d1);
+    GradJobs jobs = {{{g->a2, g->d3, GN_H, GN_H, 0, GN_H / 64, GO_W3, GO_B3},
+                      {g->a1, g->d2, GN_H, GN_H, 0, GN_H / 64, GO_W2, GO_B2},
+                      {X, g->d1, GN_IN, GN_H, 0, GN_H / 64, GO_W1, GO_B1},
+                      {g->a3, g->dout, GN_H, GN_OUT, 0, 1, GO_W4, GO_B4}}};
+    int tiles = 0;
+    for (GradJob& J : jobs.j) {
+        J.first = tiles;
+        tiles += (J.K + 63) / 64 * J.jt;
+    }
+    const int cl = grad_chunk(B), ng = (B + cl - 1) / cl;
+    k_grad_part<<<dim3(tiles, ng), b, 0, st>>>(B, cl, jobs, g->part);
+    k_sum_chunks<<<(GN_PARAMS + 255) / 256, 256, 0, st>>>(ng, GN_PARAMS, g->part, g->g);
     k_loss_sum<<<1, 1, 0, st>>>(nc, g->lpart, B, g->lpart + nc);
 }
 
@@ -672,9 +708,9 @@ extern "C" dirac_status dirac_guess_create(int max_batch, dirac_guess** out)
     al(&g->wb, (size_t)GN_IN * GN_H + 2 * GN_H * GN_H + GN_H * 8);
     al(&g->wt, (size_t)guess_tc05_packed());
     al(&g->err, 1);
-    al(&g->a1, act); al(&g->a2, act); al(&g->a3, act); al(&g->d1, act); al(&g->d2, act);
+    al(&g->a1, act); al(&g->a2, act); al(&g->a3, act); al(&g->d1, act); al(&g->d2, act); al(&g->d3, act);
     al(&g->out, (size_t)max_batch * GN_OUT); al(&g->dout, (size_t)max_batch * GN_OUT);
-    al(&g->part, (size_t)nc * GN_H * GN_H); al(&g->lpart, (size_t)nc + 1);
+    al(&g->part, (size_t)std::min(GPARTS, (max_batch + GK - 1) / GK) * GN_PARAMS); al(&g->lpart, (size_t)nc + 1);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&g->hloss, sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(g->wb, 0, sizeof(__nv_bfloat16) * ((size_t)GN_IN * GN_H + 2 * GN_H * GN_H + GN_H * 8));
     if (e == cudaSuccess) e = cudaMemset(g->wt, 0, sizeof(__nv_bfloat16) * (size_t)guess_tc05_packed());
@@ -697,7 +733,7 @@ extern "C" void dirac_guess_free(dirac_guess* g)
     if (!g) return;
     cudaDeviceSynchronize();
     for (void* p : {(void*)g->w, (void*)g->wr, (void*)g->wb, (void*)g->wt, (void*)g->err, (void*)g->m, (void*)g->v, (void*)g->g, (void*)g->a1,
-                    (void*)g->a2, (void*)g->a3, (void*)g->out, (void*)g->d1, (void*)g->d2, (void*)g->dout,
+                    (void*)g->a2, (void*)g->a3, (void*)g->out, (void*)g->d1, (void*)g->d2, (void*)g->d3, (void*)g->dout,
                     (void*)g->part, (void*)g->lpart})
         cudaFree(p);
     cudaFreeHost(g->hloss);
