@@ -299,7 +299,7 @@ void residual_accurate(dirac_op* op, const void* psi)
         }
         {
             PhaseScope ps(op, DIRAC_PHASE_VECTOR, 1);
-            k_bnorm_if<<<1, 1024, 0, op->st>>>(K.ks, op->need_b, np32, op->part_n2);
+            k_bnorm_if<<<1, finish_threads(np32), 0, op->st>>>(K.ks, op->need_b, np32, op->part_n2);
         }
         finish(op, K.ks, 1, np, nullptr, op->part_n, op->opts.max_iter);
         return;
@@ -327,7 +327,7 @@ void residual_accurate(dirac_op* op, const void* psi)
         }
         {
             PhaseScope ps(op, DIRAC_PHASE_VECTOR, 1);
-            k_bnorm_if<<<1, 1024, 0, op->st>>>(K.ks, op->need_b, op->nparts_own, op->part_n2);
+            k_bnorm_if<<<1, finish_threads(op->nparts_own), 0, op->st>>>(K.ks, op->need_b, op->nparts_own, op->part_n2);
         }
         finish(op, K.ks, 1, op->nparts_own, nullptr, op->part_n, op->opts.max_iter);
         return;
@@ -397,7 +397,7 @@ int prec_parts(const dirac_op* op, const Krylov& K)
 void finish(dirac_op* op, KState* ks, int what, int np, const double2* pd, const double* pn, int max_iter)
 {
     PhaseScope ps(op, DIRAC_PHASE_VECTOR, 1);
-    k_finish64<<<1, 1024, 0, op->st>>>(what, ks, np, pd, pn, nullptr, nullptr, max_iter);
+    k_finish64<<<1, finish_threads(np), 0, op->st>>>(what, ks, np, pd, pn, nullptr, nullptr, max_iter);
 }
 
 void vcopy(dirac_op* op, const Krylov& K, const void* a, void* b)

@@ -93,6 +93,7 @@ __global__ void k_lincomb64(int64_t n, double c0, const double2* a, double c1, c
 __global__ void k_finish64(int what, KState* st, int np, const double2* pd, const double* pn, const double2* pd2,
                            const double* pn2, int max_iter);
 __global__ void k_set_time(double* t_eval, double t);
+int finish_threads(int np);   // threads of a finisher's one block (k_finish64, k_bnorm_if)
 __global__ void k_bnorm_if(KState* st, int* flag, int np, const double* pn);
 __global__ void k_set_int(int* p, int v);
 __global__ void k_set_step_time(double* t_eval, double t_start, int step, double dt, double t_off);

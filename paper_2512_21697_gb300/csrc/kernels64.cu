@@ -157,26 +157,47 @@ __global__ void k_lincomb64(int64_t n, double c0, const double2* a, double c1, c
 // ---------------------------------------------------------------------------------------------
 // Finishers: one block sums the partials in a fixed order and advances the scalar recurrence.
 // ---------------------------------------------------------------------------------------------
+// The sums of the tree that 1024 threads would add: the levels above the partials at hand only add zeros and
+// are left out (so is a part that the caller has not got), and the last five are one warp's.  np uniform.
 __device__ void block_sum_fixed(int np, const double2* pd, const double* pn, double2* od, double* on)
 {
     __shared__ double sx[1024], sy[1024], sn[1024];
-    int t = threadIdx.x;
+    const int t = threadIdx.x;
     double ax = 0, ay = 0, an = 0;
     for (int i = t; i < np; i += blockDim.x) {
         if (pd) { ax += pd[i].x; ay += pd[i].y; }
         if (pn) an += pn[i];
     }
-    sx[t] = ax; sy[t] = ay; sn[t] = an;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (t < w) { sx[t] += sx[t + w]; sy[t] += sy[t + w]; sn[t] += sn[t + w]; }
+    int w = blockDim.x / 2;
+    while (w >= 32 && w >= np) w >>= 1;
+    if (w >= 32) {
+        sx[t] = ax; sy[t] = ay; sn[t] = an;
         __syncthreads();
+        for (; w >= 32; w >>= 1) {
+            if (t < w) {
+                if (pd) { sx[t] += sx[t + w]; sy[t] += sy[t + w]; }
+                if (pn) sn[t] += sn[t + w];
+            }
+            __syncthreads();
+        }
+        if (t < 32) { ax = sx[t]; ay = sy[t]; an = sn[t]; }
+    }
+    if (t >= 32) return;
+    for (int o = 16; o > 0; o >>= 1) {
+        if (pd) {
+            ax += __shfl_down_sync(0xffffffffu, ax, o);
+            ay += __shfl_down_sync(0xffffffffu, ay, o);
+        }
+        if (pn) an += __shfl_down_sync(0xffffffffu, an, o);
     }
     if (t == 0) {
-        if (od) *od = make_double2(sx[0], sy[0]);
-        if (on) *on = sn[0];
+        if (od) *od = make_double2(ax, ay);
+        if (on) *on = an;
     }
 }
+
+// threads of the finishers' block: up to 256 partials need no more
+int finish_threads(int np) { return np <= 256 ? 256 : 1024; }
 
 __device__ __forceinline__ bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 
@@ -204,8 +225,10 @@ __global__ void k_finish64(int what, KState* st, int np, const double2* pd, cons
 {
     __shared__ double2 d1;
     __shared__ double n1;
+    // the scalars are read beside the partials: read where they are used, each is a wait of its own
+    KState k{};
+    if (threadIdx.x == 0) k = *st;
     block_sum_fixed(np, pd, pn, &d1, &n1);
-    __syncthreads();
     if (threadIdx.x) return;
     if (what == 0) {
         st->bnorm2 = n1;
@@ -219,39 +242,39 @@ __global__ void k_finish64(int what, KState* st, int np, const double2* pd, cons
         st->rho = make_double2(n1, 0);
         st->alpha = st->omega = st->rho_prev = make_double2(1, 0);
         st->beta = make_double2(0, 0);
-        st->done = (n1 <= st->tol2 * st->bnorm2) ? 1 : 0;
+        st->done = (n1 <= k.tol2 * (what == 8 ? n1 : k.bnorm2)) ? 1 : 0;
         if (!isfinite(n1)) { st->status = 6; st->done = 1; }
         return;
     }
-    if (st->status) return;
-    if (what == 5 && st->done == 2) { st->done = 1; return; }   // the s-check finished the solve
-    if (st->done) return;
+    if (k.status) return;
+    if (what == 5 && k.done == 2) { st->done = 1; return; }   // the s-check finished the solve
+    if (k.done) return;
     if (what == 2) {
         double2 rv = d1;
         if (!finite2(rv)) { st->status = 6; st->done = 1; return; }
         if (rv.x == 0 && rv.y == 0) { st->status = 5; st->done = 1; return; }
-        st->alpha = cdiv(st->rho, rv);
+        st->alpha = cdiv(k.rho, rv);
     } else if (what == 3) {
         st->snorm2 = n1;
         if (!isfinite(n1)) { st->status = 6; st->done = 1; return; }
-        if (n1 <= st->tol2 * st->bnorm2) { st->done = 2; st->rnorm2 = n1; st->it++; }
+        if (n1 <= k.tol2 * k.bnorm2) { st->done = 2; st->rnorm2 = n1; st->it = ++k.it; }
     } else if (what == 6) {
         double2 ts = make_double2(d1.x, -d1.y);   // <t, s> = conj(<s, t>)
         double tt = n1;
         if (!(tt > 0) || !finite2(ts)) { st->status = tt == 0 ? 5 : 6; st->done = 1; return; }
         st->omega = make_double2(ts.x / tt, ts.y / tt);
     } else if (what == 5) {
-        st->it++;
+        st->it = ++k.it;
         st->rnorm2 = n1;
         if (!isfinite(n1) || !finite2(d1)) { st->status = 6; st->done = 1; return; }
-        st->rho_prev = st->rho;
+        st->rho_prev = k.rho;
         st->rho = d1;
-        if (n1 <= st->tol2 * st->bnorm2) { st->done = 1; return; }
-        if ((st->rho.x == 0 && st->rho.y == 0) || (st->omega.x == 0 && st->omega.y == 0)) {
+        if (n1 <= k.tol2 * k.bnorm2) { st->done = 1; return; }
+        if ((d1.x == 0 && d1.y == 0) || (k.omega.x == 0 && k.omega.y == 0)) {
             st->status = 5; st->done = 1; return;
         }
-        st->beta = cmul(cdiv(st->rho, st->rho_prev), cdiv(st->alpha, st->omega));
-        if (st->it >= max_iter) { st->status = 4; st->done = 1; }
+        st->beta = cmul(cdiv(d1, k.rho), cdiv(k.alpha, k.omega));
+        if (k.it >= max_iter) { st->status = 4; st->done = 1; }
     }
 }
 
