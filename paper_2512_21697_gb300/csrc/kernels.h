@@ -7,6 +7,41 @@
 
 namespace dg {
 
+// |v_u^T x|^2 of four vectors u = v .. v + 3 (the last one v1 - 1) by one warp: lane 8 u' holds vector v + u'.
+// Bound by the FP64 unit (16 cycles a warp's operation); the four pairs of sums meet in 9 additions per lane,
+// each exchange halving the values a lane is left with, where one vector's shuffle tree takes 10.
+__device__ __forceinline__ double project4(const double* __restrict__ vec, int v, int v1, int ns, const double2* x, int lane)
+{
+    const double* w[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) w[u] = vec + (int64_t)min(v + u, v1 - 1) * ns;
+    double p[8] = {};   // (re, im) of each vector's projection
+    for (int i = lane; i < ns; i += 32) {
+        const double2 xi = x[i];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const double wi = w[u][i];
+            p[2 * u] += wi * xi.x;
+            p[2 * u + 1] += wi * xi.y;
+        }
+    }
+#pragma unroll
+    for (int o = 16, m = 4; m >= 1; o >>= 1, m >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int j = 0; j < m; j++) {
+            const double keep = hi ? p[m + j] : p[j], send = hi ? p[j] : p[m + j];
+            p[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    p[0] += __shfl_xor_sync(0xffffffffu, p[0], 2);
+    p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
+    // lane bits 4, 3: the vector; bit 2: re or im
+    double q2 = p[0] * p[0];
+    q2 += __shfl_xor_sync(0xffffffffu, q2, 4);
+    return q2;
+}
+
 // Sum a (complex, real) pair over the block in a fixed order and store the block's partials.
 // Every thread of the block must call it.  Block size must be a multiple of 32, <= 1024.  A part
 // whose output is NULL is not reduced (FP64 adds are scarce on this part: a norm-only reduction

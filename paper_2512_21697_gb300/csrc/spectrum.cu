@@ -12,10 +12,10 @@
 //
 // The eigenpairs depend on kappa and the window only: computed once per window (cuSOLVER, see
 // eig_window) and kept on the device.  Three kernels per call:
-//   k_spec_proj     block per channel: S Psi_ch in shared memory, a warp per eigenvector forms the
-//                   projection (fixed shuffle tree) and stores |.|^2;
+//   k_spec_proj     block per channel: S Psi_ch in shared memory, a warp forms the projections on four
+//                   eigenvectors at a time (fixed shuffle tree) and stores |.|^2;
 //   k_spec_density  thread per level: the sum over the kappa's channels (ascending) / dE_j;
-//   k_spec_grid     thread per grid point: the interpolated densities summed over kappa.
+//   k_spec_grid     thread per (grid point, kappa): the interpolated densities, summed over kappa in order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -90,19 +90,11 @@ __global__ void k_spec_proj(OpView A, const double2* __restrict__ psi, const dou
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int v0 = vstart[ks], v1 = vstart[ks + 1];
     double* qc = q + choff[ch];
-    for (int v = v0 + warp; v < v1; v += nw) {
-        const double* w = vec + (int64_t)v * ns;
-        double2 pr = make_double2(0, 0);
-        for (int i = lane; i < ns; i += 32) {
-            const double wi = w[i];
-            pr.x += wi * sx[i].x;
-            pr.y += wi * sx[i].y;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            pr.x += __shfl_down_sync(0xffffffffu, pr.x, o);
-            pr.y += __shfl_down_sync(0xffffffffu, pr.y, o);
-        }
-        if (lane == 0) qc[v - v0] = pr.x * pr.x + pr.y * pr.y;
+    // 94 -> 83 us at 144 channels, 302 slots, 191 levels against one vector per warp at a time
+    for (int v = v0 + 4 * warp; v < v1; v += 4 * nw) {
+        const double q2 = project4(vec, v, v1, ns, sx, lane);
+        const int u = v + (lane >> 3);
+        if ((lane & 7) == 0 && u < v1) qc[u - v0] = q2;
     }
 }
 
@@ -125,19 +117,25 @@ __global__ void k_spec_density(int nvec, const double* __restrict__ E, const int
     dens[v] = sum / dE;
 }
 
-__global__ void k_spec_grid(int ngrid, const double* __restrict__ grid, int nk2, const double* __restrict__ E,
-                            const int* __restrict__ vstart, const double* __restrict__ dens, double* __restrict__ P)
+// SG_P grid points x SG_K kappas per block: a thread finds one kappa's density at one point (a chain of
+// dependent loads and a division), then the points' threads add them in ascending kappa.  47 -> 7 us at
+// 2000 points and 16 kappas, where one thread per point went through the kappas in turn.
+constexpr int SG_P = 16, SG_K = 16;
+
+__global__ void __launch_bounds__(SG_P * SG_K) k_spec_grid(int ngrid, const double* __restrict__ grid, int nk2,
+                                                           const double* __restrict__ E,
+                                                           const int* __restrict__ vstart,
+                                                           const double* __restrict__ dens, double* __restrict__ P)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= ngrid) return;
-    const double x = grid[g];
-    double acc = 0.0;
-    for (int ks = 0; ks < nk2; ks++) {
+    __shared__ double term[SG_K][SG_P];
+    const int p = threadIdx.x % SG_P, kq = threadIdx.x / SG_P, g = blockIdx.x * SG_P + p;
+    const double x = g < ngrid ? grid[g] : 0.0;
+    auto density = [&](int ks) -> double {
         const int v0 = vstart[ks], m = vstart[ks + 1] - v0;
-        if (m < 2) continue;
+        if (m < 2) return 0.0;
         const double* Ek = E + v0;
         const double* dk = dens + v0;
-        if (!(x >= Ek[0] && x <= Ek[m - 1])) continue;
+        if (!(x >= Ek[0] && x <= Ek[m - 1])) return 0.0;
         // the last level j with Ek[j] <= x (binary search over ascending levels)
         int lo = 0, hi = m - 1;
         while (lo < hi) {
@@ -145,14 +143,19 @@ __global__ void k_spec_grid(int ngrid, const double* __restrict__ grid, int nk2,
             if (Ek[mid] <= x) lo = mid;
             else hi = mid - 1;
         }
-        if (lo == m - 1) {
-            acc += dk[m - 1];
-        } else {
-            const double w = (x - Ek[lo]) / (Ek[lo + 1] - Ek[lo]);
-            acc += dk[lo] + w * (dk[lo + 1] - dk[lo]);
-        }
+        if (lo == m - 1) return dk[m - 1];
+        const double w = (x - Ek[lo]) / (Ek[lo + 1] - Ek[lo]);
+        return dk[lo] + w * (dk[lo + 1] - dk[lo]);
+    };
+    double acc = 0.0;
+    for (int k0 = 0; k0 < nk2; k0 += SG_K) {
+        term[kq][p] = g < ngrid && k0 + kq < nk2 ? density(k0 + kq) : 0.0;
+        __syncthreads();
+        if (kq == 0)
+            for (int k = 0; k < SG_K; k++) acc += term[k][p];
+        __syncthreads();
     }
-    P[g] = acc;
+    if (kq == 0 && g < ngrid) P[g] = acc;
 }
 
 #define SPTRY(call)                                                                                \
@@ -282,7 +285,7 @@ extern "C" dirac_status dirac_spectrum(dirac_op* op, const void* psi_dev, double
     }
     if (n_grid > 0) {
         SPTRY(cudaMemcpyAsync(s->grid, e_grid, sizeof(double) * n_grid, cudaMemcpyHostToDevice, op->st));
-        k_spec_grid<<<grid_for(n_grid, 128), 128, 0, op->st>>>(n_grid, s->grid, s->nvec > 0 ? s->nk2 : 0, s->E,
+        k_spec_grid<<<grid_for(n_grid, SG_P), SG_P * SG_K, 0, op->st>>>(n_grid, s->grid, s->nvec > 0 ? s->nk2 : 0, s->E,
                                                                s->vstart, s->dens, s->P);
         op->launches++;
         SPTRY(cudaGetLastError());
