@@ -883,7 +883,9 @@ __global__ void __launch_bounds__(256) k_split_rows(int n1, int NP, const double
                 b = make_float4(c.x, d.x, c.y, d.y);
                 const float2 e = df_split_bits(p.x + y.x), f = df_split_bits(p.y + y.y);
                 a = make_float4(e.x, f.x, e.y, f.y);
-                psi32[i] = make_float2(df_split_bits(p.x).x, df_split_bits(p.y).x);
+                // rounded to nearest: the truncated hi words alone would lower ||b|| by a part of their error
+                const float2 pr = df_split_bits(p.x), pi = df_split_bits(p.y);
+                psi32[i] = make_float2(pr.x + pr.y, pi.x + pi.y);
             } else {
                 const float2 e = df_split_bits(p.x), f = df_split_bits(p.y);
                 a = make_float4(e.x, f.x, e.y, f.y);

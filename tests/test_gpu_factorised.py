@@ -74,6 +74,21 @@ def test_mixed_products_match_oracle_rows(oracle_mod, kmax, N, lmax):
         assert abs(bn - torch.linalg.norm(y).item()) <= 1e-6 * bn
 
 
+# ||b|| of the factorised residual: psi rounded to nearest.  Truncated words are low by 2^-24 of a word's leading
+# bit, uniform, so by 2^-25 / mean leading fraction = 4.3e-8 on average, which is all of the bar.
+@pytest.mark.parametrize("kmax,N,lmax", [(20, 128, 1), (14, 256, 2)])
+def test_mixed_bnorm_has_no_truncation_bias(oracle_mod, kmax, N, lmax):
+    import torch
+    cfg, bas, orc, perm, inv, rows, psi = _case(oracle_mod, kmax, N, lmax, 65)
+    op = B.Operator(bas, cfg, tol=1e-10, precision=2, tol_inner=1e-5, max_outer=20)
+    pd = torch.from_numpy(psi[inv]).cuda()
+    t = 0.43 * cfg["n_cycles"] * 2 * math.pi / cfg["omega"]
+    r, y = torch.empty_like(pd), torch.empty_like(pd)
+    bn = op.residual(t, pd, pd, r)
+    op.apply(-1, t, pd, y)
+    assert abs(bn - torch.linalg.norm(y).item()) <= 4.3e-8 * bn
+
+
 # sizes where the FP64 products are factorised too (precision 0), beside the stored ones of precision 1
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("kmax,N,lmax", [(30, 96, 2), (20, 255, 2)])
