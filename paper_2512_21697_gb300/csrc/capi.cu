@@ -357,8 +357,8 @@ void k_precond_launch(dirac_op* op, const Krylov& K, int mode, const KState* ks,
 {
     PhaseScope ps(op, DIRAC_PHASE_PRECOND, 1);
     // schedule picked at setup: one lane per channel (channels of one kappa share the factor rows),
-    // one warp per channel, or one warp per channel with the vector and the factor rows staged
-    // through shared memory
+    // one warp per channel, one warp per channel with the vector and the factor rows staged through
+    // shared memory, or 16 or 32 lanes per channel with each row fixed to a lane
     if (K.prec == 1) {
         if (op->prec_sched32 == 0 && op->prec_warps)
             launch_precond_lanes_t<float>(op->prec_warps, op->st, op->ov, K.Urow, K.L, K.Dinv, op->wks, op->wfirst,
@@ -628,9 +628,8 @@ extern "C" int64_t dirac_op_device_bytes(const dirac_op* op) { return op ? (int6
 
 // Preconditioner schedules, picked by timing: one lane per channel (the channels of one kappa share
 // the factor rows read through shared memory), one warp per channel (more parallelism along the
-// band), one warp per channel with the vector and factor rows staged through shared memory, or one
-// warp per channel with each row fixed to a lane (one shuffle round per row, factor chunks only in
-// shared memory).
+// band), one warp per channel with the vector and factor rows staged through shared memory, or 16 or
+// 32 lanes per channel with each row fixed to a lane (one shuffle round per row, factors in registers).
 // Which is fastest depends on the channel count and radial size, so the operator times one
 // application of each on zeroed vectors (after a warm-up) and keeps the fastest, for the complex64
 // inner solve and for the complex128 solve.  The choice does not change results beyond the solver

@@ -60,7 +60,7 @@ struct dirac_op {
     bool split64 = false;        // the FP64 apply is split over the partners (k_apply_split)
     int prec_warps = 0;          // same-kappa channel groups (lane-per-channel preconditioner)
     // preconditioner schedules, picked by timing at setup: 0 one lane per channel (complex64 only),
-    // 1 one warp per channel, 2 one warp per channel with shared-memory staging
+    // 1 one warp per channel, 2 one warp per channel with shared-memory staging, 3 rows fixed to lanes
     int prec_sched32 = 0, prec_sched64 = 1;
     bool prec_sm_ok = false;     // the staged kernel fits this radial size
     bool prec_rot_ok = false;    // the rotated-lane kernel is set up (band width 13)
