@@ -401,15 +401,17 @@ __global__ void __launch_bounds__(128) k_precond(OpView A, const c2<T>* __restri
             if (lane == kb) w = (j + kb + 1 < n) ? zc[j + kb + 1] : mk<T>(0, 0);
         }
         __syncwarp();
-        // backward: lane k (1..wu) holds the partial sum of row i - k; the row of U for the next
-        // step is loaded one step ahead
+        // backward: lane k (1..wl) holds the partial sum of row i - k; the row of U for the next
+        // step is loaded one step ahead.  Orders from 9 on store more superdiagonals than a warp has
+        // lanes; those from 32 on are zero (checked at setup), so a row's sum starts in lane 31.
+        const int wl = min(wu, 31);
         pre_scale<T>(zc, Dk, n, lane);
-        c2<T> acc = lane >= 1 && lane <= wu ? back_start<T>(zc, n - lane) : mk<T>(0, 0);
-        c2<T> unext = (lane >= 1 && lane <= wu && n - 1 - lane >= 0) ? Uk[(int64_t)(n - 1) * (wu + 1) + lane]
+        c2<T> acc = lane >= 1 && lane <= wl ? back_start<T>(zc, n - lane) : mk<T>(0, 0);
+        c2<T> unext = (lane >= 1 && lane <= wl && n - 1 - lane >= 0) ? Uk[(int64_t)(n - 1) * (wu + 1) + lane]
                                                                       : mk<T>(0, 0);
         for (int i = n - 1; i >= 0; i--) {
             c2<T> ucur = unext;
-            if (i > 0) unext = (lane >= 1 && lane <= wu && i - 1 - lane >= 0) ? Uk[(int64_t)(i - 1) * (wu + 1) + lane]
+            if (i > 0) unext = (lane >= 1 && lane <= wl && i - 1 - lane >= 0) ? Uk[(int64_t)(i - 1) * (wu + 1) + lane]
                                                                               : mk<T>(0, 0);
             // row i is complete in lane 1; lane 0 finishes it with the reciprocal diagonal
             c2<T> a0 = shfl2<T>(acc, 1);
@@ -422,8 +424,8 @@ __global__ void __launch_bounds__(128) k_precond(OpView A, const c2<T>* __restri
             xi = shfl2<T>(xi, 0);
             // slide: lane k takes the sum of row (i-1) - k from lane k + 1, then adds U[i-k][k] x[i]
             acc = shfl2_down<T>(acc, 1);
-            if (lane == wu) acc = back_start<T>(zc, i - wu);
-            if (lane >= 1 && lane <= wu) add_back<T>(acc, ucur, xi);
+            if (lane == wl) acc = back_start<T>(zc, i - wl);
+            if (lane >= 1 && lane <= wl) add_back<T>(acc, ucur, xi);
         }
     }
     if (part_nrm) {
