@@ -188,14 +188,16 @@ dirac_status dirac_observables(dirac_op* op, const void* psi_dev, double* out, i
 dirac_status dirac_apply_assembled(dirac_op* op, int sign, const void* x_dev, void* y_dev);
 
 /* The operator of the mixed-precision inner solve alone: y = A_sign(t) x (Eq. solPsi with the
- * coupling of Eq. fullH) in complex64 arithmetic, exactly as the inner BiCGSTAB applies it --
- * FP32 copies of S and H0 per kappa, FP32 coupling values (precision 1: the FP32 rounding of the
- * FP64 assembly; precision 2: the hi words of the double-float assembly), and the kernel the
- * solve uses: the owner/gather passes for order-7 splines, the factorised apply when
- * dirac_op_set_factorised is on, else the per-row kernel; on large precision-2 systems (order 7;
- * from about 150 channels at N = 1000 or 400 at N = 250 on, all mu) the factorised product with the angular sums first, which steps
- * at tolerances below 1e-11 use, too, while those above keep the forms named before.  Assembles the coupling values for t
- * first.  x_dev, y_dev: device complex64[n] (interleaved re, im floats, library order), must not
+ * coupling of Eq. fullH) in complex64 arithmetic: FP32 copies of S and H0 per kappa, FP32 coupling
+ * values (precision 1: the FP32 rounding of the FP64 assembly; precision 2: the hi words of the
+ * double-float assembly), and the kernel the inner BiCGSTAB uses: the owner/gather passes for
+ * order-7 splines, the factorised apply when dirac_op_set_factorised is on, else the per-row kernel.
+ * On large precision-2 systems (order 7; from about 150 channels at N = 1000 or 400 at N = 250 on,
+ * all mu) the call takes the factorised product with the angular sums first, which is several times
+ * as fast there; steps use it at tolerances below 1e-11 and keep the forms named before at 1e-11 and
+ * above.  dirac_op_set_call_form(op, 1) makes the call take the steps' form at every tolerance.
+ * Assembles the coupling values for t first.  x_dev, y_dev: device complex64[n] (interleaved re, im
+ * floats, library order), must not
  * alias.  Synchronises the op's stream (it reads the error word of the bounded bulk-copy waits).
  * Errors: DIRAC_E_ARG (NULL, aliasing, sign not +-1, precision 0), DIRAC_E_CUDA. */
 dirac_status dirac_apply32(dirac_op* op, int sign, double t, const void* x_dev, void* y_dev);
@@ -205,11 +207,12 @@ dirac_status dirac_apply32(dirac_op* op, int sign, double t, const void* x_dev, 
  * to FP32.  r_dev, z_dev: device complex64[n], must not alias.  DIRAC_E_ARG for precision 0. */
 dirac_status dirac_precond_apply32(dirac_op* op, const void* r_dev, void* z_dev);
 
-/* The refinement residual of a step, r = A_-(t) psi - A_+(t) x (Eq. solPsi), computed as the step
- * computes it: precision 2 in double-float by the owner/gather passes (order-7 splines) or the
- * per-row residual kernel, precision 0 and 1 in FP64 (b = A_- psi, then r = b - A_+ x).  On large
- * precision-2 systems (see dirac_apply32) the product has the angular sums first; a step at a
- * tolerance of 1e-11 or above still takes the owner/gather passes, whose rounding error is the larger.
+/* The refinement residual of a step, r = A_-(t) psi - A_+(t) x (Eq. solPsi): precision 2 in
+ * double-float by the owner/gather passes (order-7 splines) or the per-row residual kernel, precision
+ * 0 and 1 in FP64 (b = A_- psi, then r = b - A_+ x).  On large precision-2 systems (see dirac_apply32)
+ * the call takes the product with the angular sums first, whose rounding error is the smaller, and a
+ * step at a tolerance of 1e-11 or above the owner/gather passes: dirac_op_set_call_form(op, 1) makes
+ * the call compute the residual as the step computes it.
  * Assembles the coupling values for t first.  psi_dev, x_dev, r_dev: device complex128[n]; r_dev
  * must alias neither.  bnorm (host, nullable) receives ||A_- psi||_2 as the step's tolerance test
  * uses it (precision 2: from FP32 products).  Synchronises the op's stream.  Errors: DIRAC_E_ARG,
@@ -351,10 +354,30 @@ int dirac_op_get_schedule(const dirac_op* op, int complex64);   /* -1 for a NULL
  * host and allocates the products of two radial tiles (2 x channels x multipoles x 4 x 64 x 2
  * complex64) and, for form 1, the FP32 hi words of the radial bands (written by every later
  * assembly) and the subgroup item tables.  Where a product has the angular sums first (large systems,
- * see dirac_apply32) modes 0 and 1 take it alike.  DIRAC_E_ARG for other precisions, spline orders or
+ * see dirac_apply32: single calls unless dirac_op_set_call_form, and steps below 1e-11) modes 0 and 1
+ * take it alike.  DIRAC_E_ARG for other precisions, spline orders or
  * modes; DIRAC_E_CUDA if the subgroup form's shared-memory need exceeds the device's limit.  The
  * input and output vectors of an apply must not alias. */
 dirac_status dirac_op_set_factorised(dirac_op* op, int enable);
+
+/* The form of the single products dirac_apply, dirac_apply32 and dirac_residual: as_steps = 0 (the
+ * default) the fastest form set up for the op, 1 the form its steps use, so that a call looks at the
+ * arithmetic of a step (the two differ on large precision-2 systems at tolerances of 1e-11 and above
+ * only; see dirac_apply32).  dirac_apply_assembled follows the call that assembled.  DIRAC_E_ARG for a
+ * NULL op or other values. */
+dirac_status dirac_op_set_call_form(dirac_op* op, int as_steps);
+
+/* The kernels of the op's products in the most recent call that assembled (dirac_apply,
+ * dirac_apply32, dirac_residual, dirac_step, dirac_run, dirac_solve_batch; before any: those of a
+ * step), under the current settings: product 0 the accurate operator apply, 1 the residual, 2 the
+ * complex64 apply.  -1 for a NULL op, other products, or product 2 in precision 0. */
+#define DIRAC_FORM_ROWS 0      /* stored coupling values, one thread per row */
+#define DIRAC_FORM_SPLIT 1     /* stored, the partners of a row dealt to several threads (FP64) */
+#define DIRAC_FORM_OWNER 2     /* stored, owner and gather passes */
+#define DIRAC_FORM_SUBGROUP 3  /* band products combined per subgroup (dirac_op_set_factorised 1) */
+#define DIRAC_FORM_CHANNEL 4   /* band products combined per channel (dirac_op_set_factorised 2) */
+#define DIRAC_FORM_ANGULAR 5   /* factorised, angular sums first */
+int dirac_op_get_form(const dirac_op* op, int product);
 
 /* Self-test of the bounded waits of the owner passes (their bulk-copy rings): one block waits
  * limit_cycles SM clocks (at most 4e9, about two seconds) on an mbarrier phase that nothing

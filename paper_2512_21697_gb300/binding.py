@@ -41,6 +41,10 @@ class dirac_solver_opts(C.Structure):
                 ("precond", C.c_int)]
 
 
+# dirac_op_get_form: the kernels of a product, by DIRAC_FORM_* number
+FORMS = ("rows", "split", "owner", "subgroup", "channel", "angular")
+PRODUCTS = {"apply": 0, "residual": 1, "apply32": 2}
+
 _lib = None
 _VP, _DP, _IP = C.c_void_p, C.POINTER(C.c_double), C.POINTER(C.c_int)
 SIGNATURES = {
@@ -94,6 +98,8 @@ SIGNATURES = {
     "dirac_spectrum_error": (C.c_int, [C.c_int, _DP, _DP, _DP, C.c_double, C.c_double, _DP]),
     "dirac_op_set_factorised": (C.c_int, [_VP, C.c_int]),
     "dirac_op_get_schedule": (C.c_int, [_VP, C.c_int]),
+    "dirac_op_set_call_form": (C.c_int, [_VP, C.c_int]),
+    "dirac_op_get_form": (C.c_int, [_VP, C.c_int]),
     "dirac_last_error": (C.c_char_p, []),
 }
 
@@ -297,6 +303,17 @@ class Operator:
         """dirac_op_set_residual_mode: 0 automatic (by tolerance), 1 Dot2, 2 fixed-binade offsets."""
         _check(lib().dirac_op_set_residual_mode(self._h, int(mode)), "dirac_op_set_residual_mode")
 
+    def set_call_form(self, as_steps):
+        """dirac_op_set_call_form: apply, apply32 and residual in the form the op's steps use (True) or in
+        the fastest one (False, the default)."""
+        _check(lib().dirac_op_set_call_form(self._h, int(as_steps)), "dirac_op_set_call_form")
+
+    def form(self, product):
+        """dirac_op_get_form: the kernels of "apply", "residual" or "apply32" (one of FORMS; None if the op
+        has no such product)."""
+        f = int(lib().dirac_op_get_form(self._h, PRODUCTS[product]))
+        return FORMS[f] if f >= 0 else None
+
     def device_bytes(self):
         return lib().dirac_op_device_bytes(self._h)
 
@@ -312,7 +329,8 @@ class Operator:
         _check(lib().dirac_precond_apply32(self._h, _ptr32(r), _ptr32(z)), "dirac_precond_apply32")
 
     def residual(self, t, psi, x, r):
-        """dirac_residual: r = A_-(t) psi - A_+(t) x as the step computes it; returns ||A_- psi||."""
+        """dirac_residual: r = A_-(t) psi - A_+(t) x (as the step computes it with set_call_form(True));
+        returns ||A_- psi||."""
         bn = C.c_double(0)
         _check(lib().dirac_residual(self._h, float(t), _ptr(psi), _ptr(x), _ptr(r), C.byref(bn)), "dirac_residual")
         return bn.value

@@ -126,13 +126,39 @@ void collect_phases(dirac_op* op)
 }
 
 // ---- launch helpers ------------------------------------------------------------------------
+// The kernels of each product, by the form of the running call (use_ang): every launch goes by these, and
+// dirac_op_get_form reports them.
+static int form64(const dirac_op* op)   // precision 0 and 1
+{
+    return op->use_ang ? DIRAC_FORM_ANGULAR : op->split64 ? DIRAC_FORM_SPLIT : DIRAC_FORM_ROWS;
+}
+static int form32(const dirac_op* op)
+{
+    if (op->fact32 == 2) return DIRAC_FORM_CHANNEL;
+    if (op->use_ang) return DIRAC_FORM_ANGULAR;
+    return op->fact32 == 1 ? DIRAC_FORM_SUBGROUP : op->part_own ? DIRAC_FORM_OWNER : DIRAC_FORM_ROWS;
+}
+static int form_residual(const dirac_op* op)
+{
+    if (op->opts.precision != 2) return form64(op);
+    return op->use_ang ? DIRAC_FORM_ANGULAR : op->part_rdf ? DIRAC_FORM_OWNER : DIRAC_FORM_ROWS;
+}
+static int form_apply(const dirac_op* op)
+{
+    if (op->opts.precision != 2) return form64(op);
+    return op->use_ang ? DIRAC_FORM_ANGULAR : DIRAC_FORM_ROWS;
+}
+
 int apply_parts(const dirac_op* op, const Krylov& K)
 {
-    if (op->use_ang && (K.prec == 0 || op->fact32 != 2)) return rad_parts(K.prec, op->ov.n1, op->nrad_lanes);
-    if (K.prec == 0 && op->split64) return apply_split_parts(op->ov.nch, op->ov.n1);
-    if (K.prec == 1 && op->fact32 == 1) return grid_for(op->ov.n1, FTR) * op->nfsub;
-    if (K.prec == 1 && op->fact32 == 2) return grid_for(op->ov.n1, FTR) * op->ov.nch;
-    return (K.prec == 1 && op->part_own) ? op->nparts_own : op->nparts_apply;
+    switch (K.prec == 0 ? form64(op) : form32(op)) {
+    case DIRAC_FORM_ANGULAR: return rad_parts(K.prec, op->ov.n1, op->nrad_lanes);
+    case DIRAC_FORM_SPLIT: return apply_split_parts(op->ov.nch, op->ov.n1);
+    case DIRAC_FORM_SUBGROUP: return grid_for(op->ov.n1, FTR) * op->nfsub;
+    case DIRAC_FORM_CHANNEL: return grid_for(op->ov.n1, FTR) * op->ov.nch;
+    case DIRAC_FORM_OWNER: return op->nparts_own;
+    }
+    return op->nparts_apply;
 }
 
 void k_apply_launch(dirac_op* op, const Krylov& K, int sign, const void* x, void* y, const void* bsub,
@@ -140,28 +166,28 @@ void k_apply_launch(dirac_op* op, const Krylov& K, int sign, const void* x, void
 {
     PhaseScope ps(op, K.prec == 0 ? DIRAC_PHASE_APPLY : DIRAC_PHASE_APPLY32, 1);
     dim3 grid(op->ov.nch, grid_for(op->ov.n1, 128));
-    if (K.prec == 0 && op->use_ang) {
-        op->launches++;
+    const int form = K.prec == 0 ? form64(op) : form32(op);
+    if (form == DIRAC_FORM_ANGULAR) op->launches++;   // two
+    if (K.prec == 0 && form == DIRAC_FORM_ANGULAR)
         launch_ang64(op->st, op->ov, op->ang4, op->ang_c64, op->rad_lanes, op->nrad_lanes, op->Ed, (const double*)K.S,
                      (const double*)K.H, sign, x, op->ang_S, y, bsub, dv, pdot, pnrm, skip);
-    } else if (K.prec == 0 && op->split64)
+    else if (form == DIRAC_FORM_SPLIT)
         launch_apply_split(op->st, op->ov, (const double*)K.S, (const double*)K.H, sign, x, (const double*)K.W, y, bsub,
                            dv, pdot, pnrm, skip);
     else if (K.prec == 0)
         launch_apply_t<double>(grid, op->st, op->ov, (const double*)K.S, (const double*)K.H, sign, x,
                                (const double*)K.W, y, bsub, dv, pdot, pnrm, skip);
-    else if (op->use_ang && op->fact32 != 2) {
-        op->launches++;
+    else if (form == DIRAC_FORM_ANGULAR)
         launch_ang32(op->st, op->ov, op->ang4, op->ang_c32, op->rad_lanes, op->nrad_lanes, op->aset[op->acur].Ef,
                      (const float*)K.S, (const float*)K.H, sign, x, op->ang_S, y, bsub, dv, pdot, pnrm, skip, nullptr);
-    } else if (op->fact32 == 1)
+    else if (form == DIRAC_FORM_SUBGROUP)
         launch_fact32_sub(op->st, op->ov, op->rad_lanes, op->nrad_lanes, op->fsub, op->nfsub, op->fsub_max,
                           op->fitem_off, op->fitem_coef, op->Ghi, op->pv.L, op->S32T, op->H32T, sign, x, op->Zf, y, bsub, dv,
                           pdot, pnrm, skip);
-    else if (op->fact32 == 2)
+    else if (form == DIRAC_FORM_CHANNEL)
         launch_fact32_chan(op->st, op->ov, op->rad_chunks, op->nrad, op->Gdf, op->pv.L, (const float*)K.S,
                            (const float*)K.H, sign, x, op->Zf, op->cab_df, y, bsub, dv, pdot, pnrm, skip);
-    else if (op->part_own)
+    else if (form == DIRAC_FORM_OWNER)
         launch_apply_own32(op->st, op->ov, op->S32T, op->H32T, sign, x, (const float*)K.W, y,
                            op->part_own, bsub, dv, pdot, pnrm, skip, op->dev_err);
     else
@@ -229,7 +255,7 @@ void apply_accurate(dirac_op* op, int sign, const void* x, void* y, const void* 
         k_apply_launch(op, op->k64, sign, x, y, bsub, nullptr, nullptr, pnrm, nullptr);
         return;
     }
-    if (op->use_ang && !bsub) {
+    if (form_apply(op) == DIRAC_FORM_ANGULAR && !bsub) {
         PhaseScope ps(op, DIRAC_PHASE_APPLY, 3);
         const AsmSet& a = op->aset[op->acur];
         launch_split_rows(op->st, op->ov.nch, op->ov.n1, (const double2*)x, nullptr, op->xsplit, nullptr, nullptr,
@@ -279,7 +305,7 @@ void residual_accurate(dirac_op* op, const void* psi)
         finish(op, K.ks, 1, apply_parts(op, K), nullptr, op->part_n, op->opts.max_iter);
         return;
     }
-    if (op->use_ang) {
+    if (form_residual(op) == DIRAC_FORM_ANGULAR) {
         // factorised form: no coupling values; b = A_- psi by the complex64 product on a step's first pass
         const AsmSet& a = op->aset[op->acur];
         const int np = rad_parts(2, op->ov.n1, op->nrad_lanes), np32 = rad_parts(1, op->ov.n1, op->nrad_lanes);
@@ -304,7 +330,7 @@ void residual_accurate(dirac_op* op, const void* psi)
         finish(op, K.ks, 1, np, nullptr, op->part_n, op->opts.max_iter);
         return;
     }
-    if (op->part_rdf) {
+    if (form_residual(op) == DIRAC_FORM_OWNER) {
         // owner/gather form: each coupling block read once
         {
             const bool off = residual_offsets(op);
@@ -1468,6 +1494,9 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     return DIRAC_OK;
 }
 
+// whether a single product takes the angular sums first
+static bool call_ang(const dirac_op* op) { return op->ang && (op->ang_step || !op->call_as_steps); }
+
 extern "C" dirac_status dirac_apply(dirac_op* op, int sign, double t, const void* x_dev, void* y_dev)
 {
     if (!op || !x_dev || !y_dev || x_dev == y_dev || (sign != 1 && sign != -1)) {
@@ -1476,7 +1505,7 @@ extern "C" dirac_status dirac_apply(dirac_op* op, int sign, double t, const void
     }
     k_set_time<<<1, 1, 0, op->st>>>(op->t_eval, t);
     op->launches++;
-    op->use_ang = op->ang;
+    op->use_ang = call_ang(op);
     launch_assemble(op);
     apply_accurate(op, sign, x_dev, y_dev, nullptr, nullptr);
     return check_launch("dirac_apply");
@@ -1511,7 +1540,7 @@ extern "C" dirac_status dirac_apply32(dirac_op* op, int sign, double t, const vo
     }
     k_set_time<<<1, 1, 0, op->st>>>(op->t_eval, t);
     op->launches++;
-    op->use_ang = op->ang;
+    op->use_ang = call_ang(op);
     launch_assemble(op);
     k_apply_launch(op, op->k32, sign, x_dev, y_dev, nullptr, nullptr, nullptr, nullptr, nullptr);
     dirac_status e = check_launch("dirac_apply32");
@@ -1540,7 +1569,7 @@ extern "C" dirac_status dirac_residual(dirac_op* op, double t, const void* psi_d
     Krylov& K = op->k64;
     k_set_time<<<1, 1, 0, op->st>>>(op->t_eval, t);
     op->launches++;
-    op->use_ang = op->ang;
+    op->use_ang = call_ang(op);
     launch_assemble(op);
     vcopy(op, K, x_dev, K.x);
     // b = A_- psi and ||b||^2 (precision 2 forms both inside the residual pass), then r = b - A_+ x
@@ -1697,6 +1726,22 @@ extern "C" dirac_status dirac_op_set_factorised(dirac_op* op, int enable)
     op->fact32 = enable;
     op->config_gen++;   // captured graphs hold the other apply
     return DIRAC_OK;
+}
+
+extern "C" dirac_status dirac_op_set_call_form(dirac_op* op, int as_steps)
+{
+    if (!op || (as_steps != 0 && as_steps != 1)) {
+        set_error("dirac_op_set_call_form: bad argument (0 or 1)");
+        return DIRAC_E_ARG;
+    }
+    op->call_as_steps = as_steps != 0;
+    return DIRAC_OK;
+}
+
+extern "C" int dirac_op_get_form(const dirac_op* op, int product)
+{
+    if (!op || product < 0 || product > 2 || (product == 2 && !op->k32.ks)) return -1;
+    return product == 0 ? form_apply(op) : product == 1 ? form_residual(op) : form32(op);
 }
 
 extern "C" int dirac_op_get_schedule(const dirac_op* op, int complex64)
