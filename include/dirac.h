@@ -109,15 +109,20 @@ double dirac_angular(int kappa1, int two_mu1, int kappa2, int two_mu2, int l);
 
 /* Upload the operator for one pulse and solver setting: radial blocks, pulse matrices, pair
  * coefficients and the block-banded LU factors of M = S + i dt/2 H0, and allocate every device
- * workspace (coupling values, Krylov vectors).  cuda_stream: a cudaStream_t (NULL = legacy
- * default stream).  Device memory is reported by dirac_op_device_bytes. */
+ * workspace of the steps (coupling values, Krylov vectors).  cuda_stream: a cudaStream_t (NULL =
+ * legacy default stream).  Device memory is reported by dirac_op_device_bytes. */
 dirac_status dirac_operator_setup(const dirac_basis* basis, const dirac_pulse* pulse,
                                   const dirac_solver_opts* opts, void* cuda_stream, dirac_op** out);
 void dirac_op_free(dirac_op* op);
 int64_t dirac_op_device_bytes(const dirac_op* op);
 
 /* y = A_sign(t) x, A_+- = S +- i dt/2 H(t) (Eq. solPsi), H evaluated at time t.  Assembles the
- * coupling values for t first.  x_dev, y_dev: device complex128[n], must not alias. */
+ * coupling values for t first.  x_dev, y_dev: device complex128[n], must not alias.  On large
+ * precision-2 systems whose steps keep the stored coupling values (see dirac_apply32) the first call
+ * of dirac_apply, dirac_apply32 or dirac_residual sets up the workspace of the products with the
+ * angular sums first: it allocates (6 % of the op's memory at the production size) and synchronises
+ * the op's stream.  A call on a captured stream allocates nothing, and on a device without room for
+ * the workspace the op keeps these calls as they are: both then take the steps' form. */
 dirac_status dirac_apply(dirac_op* op, int sign, double t, const void* x_dev, void* y_dev);
 /* z = M^-1 r with M = S + i dt/2 H0 (Eq. matrixM).  r_dev, z_dev: device complex128[n]. */
 dirac_status dirac_precond_apply(dirac_op* op, const void* r_dev, void* z_dev);

@@ -759,20 +759,15 @@ static bool ang_pays(const dirac_op* op)
 // sums, the states of the two forms agree to 5e-13.
 static bool ang_steps(const dirac_op* op)
 {
-    return op->ang && (op->opts.precision != 2 || op->opts.tol < 1e-11);
+    return op->ang_pays && (op->opts.precision != 2 || op->opts.tol < 1e-11);
 }
 
-// Tables and buffers of the factorised products (kernels_ang.cu): kappa chunks of up to FLANE channels
-// for the radial pass, two per warp where they fit; for the angular pass lists of neighbouring channels
-// of one mu and one parity of the orbital l with, per multipole, the union of their partners and each
-// output's coefficients
-//   alpha = c tau A1(a, b) (of K_l(ka, kb)), beta = -c tau A2(a, b) (of KT_l(kb, ka)).
-// ord: the channels sorted by kappa slot.
-static dirac_status ang_setup(dirac_op* op, const std::vector<int>& ord, const std::vector<int>& kslot)
+// Radial passes of the factorised products: kappa chunks of up to FLANE channels, two per warp where they
+// fit.  ord: the channels sorted by kappa slot.
+static dirac_status rad_setup(dirac_op* op, const std::vector<int>& ord, const std::vector<int>& kslot)
 {
     const Basis& B = op->B;
-    const int nch = B.nch, L = op->pv.L, n1 = B.n1;
-    const double ct = B.p.c * 0.5 * op->opts.dt;
+    const int nch = B.nch;
     std::vector<RadChunk> ch1;
     for (int i = 0; i < nch;) {
         int j = i;
@@ -802,7 +797,41 @@ static dirac_status ang_setup(dirac_op* op, const std::vector<int>& ord, const s
     dirac_status e = upload(op, &op->rad_lanes, rl);
     if (e) return e;
     op->nrad_lanes = (int)rl.size();
-    if (!ang_pays(op)) return DIRAC_OK;
+    return DIRAC_OK;
+}
+
+// Band entries of a buffer set in the precisions of precision 2 (double-float with row sums, complex64).
+static dirac_status ang_bands(dirac_op* op, AsmSet& a)
+{
+    const size_t rows = (size_t)op->pv.L * 18 * op->B.n1;   // 6 sums x 3 values
+    float *Ef, *Ers;
+    float2* Ex;
+    dirac_status e = dev_alloc(op, &Ef, rows * 13);
+    if (!e) e = dev_alloc(op, &Ex, rows * 13);
+    if (!e) e = dev_alloc(op, &Ers, rows);
+    if (e) return e;
+    a.Ef = Ef; a.Ex = Ex; a.Ers = Ers;
+    return DIRAC_OK;
+}
+
+// Tables and buffers of the products with the angular sums first (kernels_ang.cu): lists of neighbouring
+// channels of one mu and one parity of the orbital l with, per multipole, the union of their partners and
+// each output's coefficients
+//   alpha = c tau A1(a, b) (of K_l(ka, kb)), beta = -c tau A2(a, b) (of KT_l(kb, ka)).
+static dirac_status ang_setup(dirac_op* op)
+{
+    const Basis& B = op->B;
+    const int nch = B.nch, L = op->pv.L, n1 = B.n1;
+    const double ct = B.p.c * 0.5 * op->opts.dt;
+    // copies on the op's stream: a single product may come here while another stream is captured
+    auto put = [&](auto** out, const auto& host) -> dirac_status {
+        dirac_status e = dev_alloc(op, out, host.size());
+        if (e || host.empty()) return e;
+        CUDA_TRY(cudaMemcpyAsync(*out, host.data(), host.size() * sizeof(host[0]), cudaMemcpyHostToDevice, op->st));
+        CUDA_TRY(cudaStreamSynchronize(op->st));
+        return DIRAC_OK;
+    };
+    dirac_status e = DIRAC_OK;
     // per (channel, multipole): (partner, alpha, beta), partners ascending within each half of the list
     struct Use { int b; double al, be; };
     std::vector<std::vector<Use>> uses((size_t)nch * L);
@@ -882,17 +911,16 @@ static dirac_status ang_setup(dirac_op* op, const std::vector<int>& ord, const s
         }
         int *dout = nullptr, *dstart = nullptr, *di = nullptr;
         float4* dcs = nullptr;
-        dirac_status e = upload(op, &dout, lout);
-        if (!e) e = upload(op, &dstart, start);
-        if (!e) e = upload(op, &di, item);
-        if (!e) e = upload(op, &dcs, csum);
+        dirac_status e = put(&dout, lout);
+        if (!e) e = put(&dstart, start);
+        if (!e) e = put(&di, item);
+        if (!e) e = put(&dcs, csum);
         v.L = L; v.nlist = (int)groups.size(); v.out = dout; v.start = dstart; v.item = di; v.csum = dcs;
         return e;
     };
     std::vector<double> coef, coefx;
     if (!e) e = lists(AG4, op->ang4, coef);
     const bool mixed = op->opts.precision == 2;   // double-float and complex64 products
-    const size_t ne = (size_t)L * 18 * n1 * 13;   // band entries: 6 sums x 3 values
     if (mixed) {
         if (!e) e = lists(AGX, op->angx, coefx);
         std::vector<float> cf(coef.begin(), coef.end());
@@ -902,29 +930,57 @@ static dirac_status ang_setup(dirac_op* op, const std::vector<int>& ord, const s
             cx[i] = make_float4(h, h, lo, lo);
         }
         if (!e) e = dev_alloc(op, &op->ang_umax, (size_t)nch * ang_np(n1));
-        if (!e) e = upload(op, &op->ang_c32, cf);
-        if (!e) e = upload(op, &op->ang_cx, cx);
-        AsmSet& a = op->aset[0];
-        if (!e) e = dev_alloc(op, &a.Ef, ne);
-        if (!e) e = dev_alloc(op, &a.Ex, ne);
-        if (!e) e = dev_alloc(op, &a.Ers, (size_t)L * 18 * n1);
+        if (!e) e = put(&op->ang_c32, cf);
+        if (!e) e = put(&op->ang_cx, cx);
+        if (!e) e = ang_bands(op, op->aset[op->acur]);
     } else {
-        if (!e) e = upload(op, &op->ang_c64, coef);
-        if (!e) e = dev_alloc(op, &op->Ed, ne);
+        if (!e) e = put(&op->ang_c64, coef);
+        if (!e) e = dev_alloc(op, &op->Ed, (size_t)L * 18 * n1 * 13);
     }
     char* S = nullptr;
     if (!e) e = dev_alloc(op, &S, ((size_t)nch * (6 * L + (mixed ? 0 : 2)) * ang_np(n1) + ang_tail()) * 16);
-    // where the steps keep the stored form, a card without room for this one still takes the operator
-    if (e == DIRAC_E_NOMEM && mixed && op->opts.tol >= 1e-11) {
-        cudaGetLastError();
-        return DIRAC_OK;
-    }
     if (e) return e;
     op->ang_S = S;
     CUDA_TRY(ang_prepare());
     op->ang = true;
-    op->ang_step = op->use_ang = ang_steps(op);
     return DIRAC_OK;
+}
+
+// Whether a single product (dirac_apply, dirac_apply32, dirac_residual) takes the angular sums first.  Where
+// the steps keep the stored form, the first such product sets the tables up (at 1860 channels, 1001 slots
+// and seven multipoles 1.3 GB beside 21.8, in 15 ms), so that an op which only steps holds none of them.
+// Nothing is allocated while the op's stream is captured, nor where memory is short: the product then takes
+// the stored form.
+static bool call_ang(dirac_op* op)
+{
+    if (op->ang_step) return true;
+    if (!op->ang_pays || op->call_as_steps || op->ang_short) return false;
+    AsmSet& a = op->aset[op->acur];
+    if (op->ang && a.Ef) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(op->st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    const size_t nalloc = op->allocs.size();
+    const auto bytes = op->bytes;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // other streams' captures stay valid
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    dirac_status e;
+    try {
+        e = op->ang ? ang_bands(op, a) : ang_setup(op);
+    } catch (const std::bad_alloc&) {
+        e = DIRAC_E_NOMEM;
+    }
+    if (e) {
+        cudaGetLastError();
+        op->ang_short = true;   // not tried again: the op's products keep one form
+        if (!op->ang) a.Ef = nullptr;
+        for (; op->allocs.size() > nalloc; op->allocs.pop_back()) cudaFree(op->allocs.back());
+        op->bytes = bytes;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e == DIRAC_OK;
 }
 
 extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dirac_pulse* pulse,
@@ -1204,7 +1260,14 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     TRY(dev_alloc(op, &op->s, (size_t)P.L * 3));
     TRY(dev_alloc(op, &op->t_eval, 1));
     op->pv.L = P.L;
-    if (bd == 13 && op->npairs) TRY(ang_setup(op, ord, kslot));   // factorised products, where they are the faster form
+    if (bd == 13 && op->npairs) {   // factorised products, where they are the faster form
+        TRY(rad_setup(op, ord, kslot));
+        op->ang_pays = ang_pays(op);
+        if (ang_steps(op)) {
+            TRY(ang_setup(op));
+            op->ang_step = op->use_ang = true;
+        }
+    }
     const size_t wlen = op->ang_step ? 1 : (size_t)std::max<int64_t>(op->npairs, 1) * be;   // stored coupling values
     if (!dfloat) {
         TRY(dev_alloc(op, &op->W, wlen));
@@ -1431,8 +1494,8 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     op->nparts_prec = grid_for(B.nch, 4);                     // ||s||^2 partials, warp-per-channel kernel
     op->nparts_prec32 = op->prec_warps ? op->prec_warps : grid_for(B.nch, 4);   // lane-per-channel kernel
     int np = std::max({op->nparts_apply, op->split64 ? apply_split_parts(B.nch, n1) : 0, op->nparts_own, op->nparts_vec, op->nparts_prec, op->nparts_prec32,
-                       grid_for(n1, FTR) * B.nch, op->ang ? rad_parts(0, n1, op->nrad_lanes) : 0,
-                       op->ang ? rad_parts(1, n1, op->nrad_lanes) : 0,
+                       grid_for(n1, FTR) * B.nch, op->ang_pays ? rad_parts(0, n1, op->nrad_lanes) : 0,
+                       op->ang_pays ? rad_parts(1, n1, op->nrad_lanes) : 0,
                        precond_sm_blocks<double>(B.nch), precond_sm_blocks<float>(B.nch),
                        precond_rot_blocks<double>(B.nch), precond_rot_blocks<float>(B.nch)});
     TRY(dev_alloc(op, &op->part_d, (size_t)np));
@@ -1493,9 +1556,6 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
 #undef TRY
     return DIRAC_OK;
 }
-
-// whether a single product takes the angular sums first
-static bool call_ang(const dirac_op* op) { return op->ang && (op->ang_step || !op->call_as_steps); }
 
 extern "C" dirac_status dirac_apply(dirac_op* op, int sign, double t, const void* x_dev, void* y_dev)
 {
@@ -1805,12 +1865,7 @@ extern "C" dirac_status dirac_op_set_overlap(dirac_op* op, int enable)
             CUDA_TRY(cudaEventCreateWithFlags(&op->ev_use[i], cudaEventDisableTiming));
         }
         if (op->aset[0].Ghi && (e = dev_alloc(op, &a.Ghi, (size_t)op->pv.L * 4 * be))) return e;
-        if (op->ang) {
-            const size_t ne = (size_t)op->pv.L * 18 * op->ov.n1 * 13;
-            if ((e = dev_alloc(op, &a.Ef, ne)) || (e = dev_alloc(op, &a.Ex, ne)) ||
-                (e = dev_alloc(op, &a.Ers, (size_t)op->pv.L * 18 * op->ov.n1)))
-                return e;
-        }
+        if (op->ang_step && (e = ang_bands(op, a))) return e;
         op->aset[1] = a;
     }
     op->overlap = enable != 0;

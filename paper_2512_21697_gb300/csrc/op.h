@@ -96,8 +96,10 @@ struct dirac_op {
     float4* fitem_coef = nullptr;        // item -> FSG coefficient sets (U, V, U', V')
     // factorised products with the angular sums first (kernels_ang.cu), the accurate and the complex64
     // ones, for systems where they are the faster form
-    bool ang = false;                    // they are set up: single products take them, unless
-    bool call_as_steps = false;          // .. the caller wants those as the steps compute them
+    bool ang_pays = false;               // this is such a system
+    bool ang = false;                    // they are set up
+    bool ang_short = false;              // no memory for that: the single products keep the stored form
+    bool call_as_steps = false;          // the caller wants single products as the steps compute them
     bool ang_step = false;               // steps take them, too: no coupling values are stored
     bool use_ang = false;                // the form of the running call, and of the last assembly
     dg::AngList ang4{}, angx{};          // lists of AG4 and of AGX outputs
