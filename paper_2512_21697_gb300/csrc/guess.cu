@@ -35,7 +35,7 @@ constexpr int GN_IN = 32, GN_H = 256, GN_OUT = 4;
 constexpr int64_t GO_W1 = 0, GO_B1 = GO_W1 + GN_IN * GN_H, GO_W2 = GO_B1 + GN_H, GO_B2 = GO_W2 + GN_H * GN_H,
                   GO_W3 = GO_B2 + GN_H, GO_B3 = GO_W3 + GN_H * GN_H, GO_W4 = GO_B3 + GN_H,
                   GO_B4 = GO_W4 + GN_H * GN_OUT, GN_PARAMS = GO_B4 + GN_OUT;
-constexpr int GCHUNK = 1024;   // samples per partial of the loss
+constexpr int GCHUNK = 1024;   // samples per partial of the loss, and at most of a gradient
 
 }  // namespace dg
 
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* 
 // Partial gradients of every layer over one chunk of clen samples (blockIdx.y), laid out as the parameters,
 // P[chunk][parameter]: a weight gradient W[k][j] = sum_i A[i][k] D[i][j] in 64 x 64 tiles (blockIdx.x over the
 // layers' tiles), and with its first row of tiles the bias gradient b[j] = sum_i D[i][j].  The four layers
-// have 40 tiles, so the samples are split into up to 32 chunks to fill the chip: 50 us for 4096 samples,
+// have 40 tiles, so the samples are split into 32 chunks (see grad_chunk) to fill the chip: 50 us for 4096 samples,
 // against 665 us for one launch per layer over chunks of 1024 and 248 us for its column sums.
 struct GradJob {
     const float *A, *D;
@@ -647,9 +647,12 @@ dirac_status gcheck(cudaError_t e, const char* what)
     } while (0)
 
 int nchunks(int B) { return (B + GCHUNK - 1) / GCHUNK; }
-// samples per partial of the parameter gradients: at most 32 partials, each of whole staged chunks
+// Samples per partial of the parameter gradients: 32 partials of whole staged chunks, and more where a
+// partial would be longer than GCHUNK samples (batches above 32768): its FP32 sum runs over them in turn, and
+// its rounding grows with their number (1048576 equal samples in 32 partials: 2.5e-4; in 1024: 1.2e-5).
 constexpr int GPARTS = 32;
-int grad_chunk(int B) { return GK * ((B + GK * GPARTS - 1) / (GK * GPARTS)); }
+int grad_chunk(int B) { return std::min(GCHUNK, GK * ((B + GK * GPARTS - 1) / (GK * GPARTS))); }
+int grad_parts(int max_batch) { return std::max(std::min(GPARTS, (max_batch + GK - 1) / GK), nchunks(max_batch)); }
 
 // forward through the FP32 kernels, keeping the activations (training and the reference path)
 void fwd32(dirac_guess* g, const float* X, int B, cudaStream_t st)
@@ -710,7 +713,7 @@ extern "C" dirac_status dirac_guess_create(int max_batch, dirac_guess** out)
     al(&g->err, 1);
     al(&g->a1, act); al(&g->a2, act); al(&g->a3, act); al(&g->d1, act); al(&g->d2, act); al(&g->d3, act);
     al(&g->out, (size_t)max_batch * GN_OUT); al(&g->dout, (size_t)max_batch * GN_OUT);
-    al(&g->part, (size_t)std::min(GPARTS, (max_batch + GK - 1) / GK) * GN_PARAMS); al(&g->lpart, (size_t)nc + 1);
+    al(&g->part, (size_t)grad_parts(max_batch) * GN_PARAMS); al(&g->lpart, (size_t)nc + 1);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&g->hloss, sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(g->wb, 0, sizeof(__nv_bfloat16) * ((size_t)GN_IN * GN_H + 2 * GN_H * GN_H + GN_H * 8));
     if (e == cudaSuccess) e = cudaMemset(g->wt, 0, sizeof(__nv_bfloat16) * (size_t)guess_tc05_packed());
