@@ -132,7 +132,7 @@ class ClockSampler:
 
 
 def operator_counts(bas, cfg, kind):
-    """Algorithmic bytes and flops of one operator apply A_+- x.
+    """Algorithmic bytes and flops of one operator apply A_+- x on stored coupling values.
 
     kind 'f64': FP64 values and vectors; 'f32': FP32 values, complex64 vectors; 'df': double-float
     values (hi + lo floats, 8 B), split input vector (16 B per complex), complex128 output.
@@ -146,6 +146,23 @@ def operator_counts(bas, cfg, kind):
     vb, ib, ob = {"f64": (8, 16, 16), "f32": (4, 8, 8), "df": (8, 16, 16)}[kind]
     bytes_ = vb * coup + (ib + ob) * bas.n + 2 * vb * nk2 * n1 * bd * 4
     return coup, flops, bytes_
+
+
+def factorised_counts(bas, cfg, form, kind):
+    """(multiply-adds by part, bytes) of one factorised apply: 'angular' (k_ang + k_rad: six angular sums per
+    channel, multipole and slot, each through two rows of bands) or the band products of the subgroup and
+    per-channel forms.  Useful multiply-adds only; real x complex counts two.  No coupling values are
+    read: the bytes are the vectors', and for 'angular' the bands' at the current time."""
+    n1, bd, L = cfg["N"] + 1, 2 * cfg["order"] - 1, cfg["l_max"] + 1
+    vb, xb = {"f64": (8, 32), "f32": (4, 16), "df": (8, 32)}[kind]
+    fma = {"diagonal": 16 * bas.nch * n1 * bd}
+    if form == "angular":
+        fma["angular"] = 2 * bas.nterms * n1 * 12
+        fma["radial"] = bas.nch * L * n1 * bd * 24
+        return fma, xb * bas.n + vb * n1 * bd * (18 * L + 2 * 2 * cfg["kappa_max"] * 4)
+    fma["angular"] = 2 * bas.nterms * n1 * 16
+    fma["radial"] = bas.nch * L * n1 * bd * 32
+    return fma, xb * bas.n
 
 
 FP32_LANE_OPS = 152 * 128 * 2.070   # 10^9 lane operations/s: SMs x FP32 lanes x max clock (GHz)
@@ -163,19 +180,24 @@ DF_OPS_PER_FMA_OFF = 6              # ... in the fixed-binade form (df_fma_off),
 OFFSET_TOL = 1e-11                  # the library picks the fixed-binade form at tolerances >= this
 
 
-def roofline_of(bas, cfg, phase, kind, ms, cnt, hbm_peak, fact=1):
+def roofline_of(bas, cfg, phase, kind, ms, cnt, hbm_peak, form):
     """Roofline of one operator-apply launch group, timed live by the library's event timers.
 
-    kind 'f64': FP64 apply (FP64 ALU bound), 'f32': complex64 owner/gather apply (HBM bound),
-    'df': double-float refinement residual pass (FP32 ALU/issue bound), 'df_owner': its owner pass.
+    kind 'f64': FP64 apply (FP64 ALU bound), 'f32': complex64 apply (HBM bound on stored values, else FP32
+    ALU), 'df': double-float refinement residual pass (FP32 ALU/issue bound), 'df_owner': its product
+    alone (the owner pass; k_ang + k_rad).  form: the kernels that ran (binding.Operator.form).
     The owner pass's coupling products take DF_OPS_PER_FMA_OFF operations at tolerances >= 1e-11
     (the library's automatic choice), DF_OPS_PER_FMA below; the gather's diagonal blocks always ten."""
-    cops = DF_OPS_PER_FMA_OFF if cfg["tol"] >= OFFSET_TOL else DF_OPS_PER_FMA
-    coup, flops, bytes_ = operator_counts(bas, cfg, {"df_owner": "df", "fact32": "f32"}.get(kind, kind))
+    cops = DF_OPS_PER_FMA_OFF if cfg["tol"] >= OFFSET_TOL and form != "rows" else DF_OPS_PER_FMA
+    counts = {"df_owner": "df"}.get(kind, kind)
+    coup, flops, bytes_ = operator_counts(bas, cfg, counts)
+    factorised = form in ("angular", "subgroup", "channel")
+    if factorised:
+        fma, bytes_ = factorised_counts(bas, cfg, form, counts)
     t = ms / cnt / 1000.0
     gbs = bytes_ / t / 1e9
     traffic, tnote = None, None
-    if kind in TRAFFIC_MEDIUM:
+    if kind in TRAFFIC_MEDIUM and form == "owner":
         units = bas.npairs * (cfg["N"] + 1)
         traffic = TRAFFIC_MEDIUM[kind][0] * units / MEDIUM_UNITS
         tnote = ("owner pass only, from %s (medium capture) scaled by pairs x radial slots (x%.3f)" %
@@ -183,37 +205,45 @@ def roofline_of(bas, cfg, phase, kind, ms, cnt, hbm_peak, fact=1):
     out = {"phase": phase, "apply_ms": t * 1000.0, "bytes_per_apply": bytes_, "gbs": gbs, "traffic": traffic}
     if tnote:
         out["traffic_note"] = tnote
+    fp32 = {"bound": "alu", "unit": "TFLOP/s", "peak": 2 * FP32_LANE_OPS / 1e3,
+            "peak_source": "derived FP32 FMA rate: 152 SMs x 128 lanes x 2 flop x 2.07 GHz"}
+    lanes = {"bound": "alu", "unit": "T FP32-lane-ops/s", "peak": FP32_LANE_OPS / 1e3,
+             "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz (1 op per lane per clock); "
+                            "%d ops per coupling multiply-add, 10 per diagonal-block one" % cops}
     if kind == "f64":
+        if factorised:
+            flops = 2 * sum(fma.values())
+            out["fma_per_apply"] = fma
         tf = flops / t / 1e12
-        out.update({"kernel": "k_apply<double> (FP64 operator apply)", "flops_per_apply": flops, "bound": "alu",
-                    "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": tf / FP64_PEAK_TFLOPS,
+        out.update({"kernel": {"rows": "k_apply<double> (FP64 operator apply)",
+                               "split": "k_apply_split (FP64 operator apply, partners dealt to several threads)",
+                               "angular": "k_ang<double> + k_rad<double> (FP64 operator apply, angular sums first)"}[form],
+                    "flops_per_apply": flops, "bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS,
+                    "unit": "TFLOP/s", "frac": tf / FP64_PEAK_TFLOPS,
                     "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"})
-    elif kind == "fact32":
-        # factorised complex64 apply: useful FMAs only (the radial band products of every channel and
-        # multipole, the angular combination of each directed pair term, the diagonal blocks); it
-        # reads no coupling values, so its HBM bytes are the vectors' and it is timed against the
-        # FP32 FMA rate (one FMA per lane per clock)
-        n1, bd = cfg["N"] + 1, 2 * cfg["order"] - 1
-        L = cfg["l_max"] + 1
-        fma_rad = bas.nch * L * n1 * 4 * 2 * bd * 2 * 2
-        fma_ang = 2 * bas.nterms * n1 * 2 * 8
-        fma_diag = bas.nch * n1 * 2 * bd * 2 * 4
-        fma = fma_rad + fma_ang + fma_diag
-        out["bytes_per_apply"] = (8 + 8) * bas.n
-        out["gbs"] = out["bytes_per_apply"] / t / 1e9
-        tf = 2 * fma / t / 1e12
-        peak = 2 * FP32_LANE_OPS / 1e3
-        out.update({"kernel": ("k_fact_tile32 (factorised complex64 inner-solve apply, subgroup form: radial pass "
-                               "of tile t+1 beside the angular pass of tile t)" if fact == 1 else
-                               "k_fact_radial32 + k_fact_angular32 (factorised complex64 inner-solve apply, "
-                               "per-channel form)"),
-                    "fma_per_apply": {"radial": fma_rad, "angular": fma_ang, "diagonal": fma_diag},
-                    "bound": "alu", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak,
-                    "peak_source": "derived FP32 FMA rate: 152 SMs x 128 lanes x 2 flop x 2.07 GHz"})
+    elif kind == "f32" and factorised:
+        # timed against the FP32 FMA rate (one FMA per lane per clock)
+        tf = 2 * sum(fma.values()) / t / 1e12
+        out.update(fp32, kernel={"subgroup": "k_fact_tile32 (factorised complex64 inner-solve apply, subgroup form: "
+                                             "radial pass of tile t+1 beside the angular pass of tile t)",
+                                 "channel": "k_fact_radial32 + k_fact_angular32 (factorised complex64 inner-solve "
+                                            "apply, per-channel form)",
+                                 "angular": "k_ang<float> + k_rad<float> (complex64 inner-solve apply, angular sums "
+                                            "first)"}[form],
+                   fma_per_apply=fma, achieved=tf, frac=tf / fp32["peak"])
     elif kind == "f32":
-        out.update({"kernel": "k_apply_own32 + k_apply_gather32 (complex64 inner-solve apply)",
+        out.update({"kernel": {"owner": "k_apply_own32 + k_apply_gather32 (complex64 inner-solve apply)",
+                               "rows": "k_apply<float> (complex64 inner-solve apply)"}[form],
                     "flops_per_apply": flops, "bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s",
                     "frac": gbs / hbm_peak})
+    elif factorised:
+        # double-float multiply-adds of k_ang and k_rad; the diagonal blocks S and tau H0 are Dot2 sums
+        dfma = sum(fma.values())
+        ops = (dfma - fma["diagonal"]) * cops + fma["diagonal"] * DF_OPS_PER_FMA
+        tops = ops / t / 1e12
+        out.update(lanes, kernel="k_ang + k_rad (double-float refinement residual, angular sums first)" +
+                   ("" if kind == "df_owner" else ", with k_split_rows and a step's complex64 norm of b"),
+                   df_fma_per_apply=dfma, ops_per_apply=ops, achieved=tops, frac=tops / lanes["peak"])
     elif kind == "df_owner":
         # the owner pass alone: it streams the hi and lo words of every stored coupling value once
         # (HBM), and forms each value's two uses (W u_b, W^T u_a) on re and im in double-float
@@ -238,32 +268,43 @@ def roofline_of(bas, cfg, phase, kind, ms, cnt, hbm_peak, fact=1):
         dfma = 4 * coup + 4 * bas.nch * n1 * bd * 4
         ops = 4 * coup * cops + 4 * bas.nch * n1 * bd * 4 * DF_OPS_PER_FMA
         tops = ops / t / 1e12
-        peak = FP32_LANE_OPS / 1e3
-        out.update({"kernel": "k_split_uv3 + k_residual_own_df + k_residual_gather_df (double-float refinement "
-                              "residual)", "df_fma_per_apply": dfma, "ops_per_apply": ops, "bound": "alu",
-                    "achieved": tops, "peak": peak, "unit": "T FP32-lane-ops/s", "frac": tops / peak,
-                    "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz (1 op per lane per clock); "
-                                   "%d ops per coupling multiply-add, 10 per diagonal-block one" % cops})
+        out.update(lanes, kernel={"owner": "k_split_uv3 + k_residual_own_df + k_residual_gather_df (double-float "
+                                           "refinement residual)",
+                                  "rows": "k_residual_df (double-float refinement residual)"}[form],
+                   df_fma_per_apply=dfma, ops_per_apply=ops, achieved=tops, frac=tops / lanes["peak"])
     return out
 
 
-def roofline(bas, cfg, phase_ms, phase_n, precision, hbm_peak, factorised=0):
-    """The dominant kernel's roofline, plus the complex64 SpMV's when it ran.  In precision 2 the
-    dominant kernel is the residual's owner pass, timed on its own (its phase lies inside 'apply');
+def roofline(bas, cfg, phase_ms, phase_n, precision, hbm_peak, forms):
+    """The dominant kernel's roofline, plus the complex64 SpMV's when it ran; forms: the kernels of the
+    "residual" and "apply32" products (binding.Operator.form).  In precision 2 the dominant kernel is the
+    residual's product (the owner pass; k_ang + k_rad), timed on its own (its phase lies inside 'apply');
     the whole residual pass (split, owner, gather) is reported beside it."""
     cands = []
     if phase_n.get("apply", 0):
-        cands.append(("apply", "df" if precision == 2 else "f64", phase_ms["apply"], phase_n["apply"]))
+        cands.append(("apply", "df" if precision == 2 else "f64", phase_ms["apply"], phase_n["apply"], forms["residual"]))
     if phase_n.get("apply32", 0):
-        cands.append(("apply32", "fact32" if factorised else "f32", phase_ms["apply32"], phase_n["apply32"]))
-    outs = {c[0]: roofline_of(bas, cfg, c[0], c[1], c[2], c[3], hbm_peak, factorised) for c in cands}
+        cands.append(("apply32", "f32", phase_ms["apply32"], phase_n["apply32"], forms["apply32"]))
+    outs = {c[0]: roofline_of(bas, cfg, c[0], c[1], c[2], c[3], hbm_peak, c[4]) for c in cands}
     dom = max(cands, key=lambda c: c[2])[0]
     if dom == "apply" and precision == 2 and phase_n.get("owner", 0):
         whole = outs["apply"]
-        own = roofline_of(bas, cfg, "owner", "df_owner", phase_ms["owner"], phase_n["owner"], hbm_peak)
+        own = roofline_of(bas, cfg, "owner", "df_owner", phase_ms["owner"], phase_n["owner"], hbm_peak, forms["residual"])
         own["residual_pass"] = {k: whole[k] for k in ("kernel", "apply_ms", "achieved", "frac")}
         return own, outs.get("apply32")
     return outs[dom], outs.get("apply32")
+
+
+STORED_FORMS = ("rows", "split", "owner")
+
+
+def l2_note(bas, cfg, forms):
+    """What an apply moves between two uses of the same data, against the L2 cache."""
+    if any(f in STORED_FORMS for f in forms.values()):
+        coup = bas.npairs * (cfg["N"] + 1) * (2 * cfg["order"] - 1) * 4
+        return "inputs larger than L2: %.1f GB of coupling values streamed per operator apply" % (8 * coup / 1e9)
+    sums = bas.nch * 6 * (cfg["l_max"] + 1) * (cfg["N"] + 1) * 16
+    return "no coupling values stored: %.2f GB of angular sums written and read per accurate operator apply" % (sums / 1e9)
 
 
 def max_over_ranks(ms, dist=None, device=None):
@@ -860,6 +901,7 @@ def main():
     ms_host = hl0.elapsed_time(hl1)
     phase_ms, phase_n, launches = op.profile_read()
     op.profile(False)
+    forms = {k: op.form(k) for k in ("residual", "apply32") if op.form(k)}   # the kernels of those steps
     tcur += args.steps * dt
 
     # end to end through the C ABI with host buffers: per step, the state in from pinned host memory,
@@ -895,15 +937,13 @@ def main():
     e2e_sps = e2e_steps / (ee0.elapsed_time(ee1) / 1000.0) * world
 
     peak_bw, peak_src = hbm_peak()
-    roof, roof32 = roofline(bas, cfg, phase_ms, phase_n, args.precision, peak_bw,
-                            args.factorised if args.precision == 2 else 0)
+    roof, roof32 = roofline(bas, cfg, phase_ms, phase_n, args.precision, peak_bw, forms)
     for r in (roof, roof32):
         if r and r["bound"] == "hbm":
             r["peak_source"] = "%s copy bandwidth %.1f GB/s" % ("measured" if peak_src == "measured" else
                                                               "fallback", peak_bw)
     roof["timing"] = ("phase events around the kernel's launches during %d host-loop steps run right after the "
                       "headline's graph-driven steps (same kernels, same window)" % args.steps)
-    coup = bas.npairs * (cfg["N"] + 1) * (2 * cfg["order"] - 1) * 4
     if rank != 0:
         if dist:
             dist.destroy_process_group()
@@ -922,14 +962,15 @@ def main():
                    "driver": ("dirac_run: the time loop as one CUDA graph with conditional WHILE/IF nodes, one "
                               "graph launch and one status read-back per call" if graph else
                               "dirac_step: host-driven loop"),
-                   "inner_apply": (["stored coupling values (owner/gather passes)",
-                                    "factorised: radial band products x angular coefficients, subgroup form",
-                                    "factorised: radial band products x angular coefficients, per-channel form"]
-                                   [args.factorised] if args.precision == 2 else None),
+                   "inner_apply": ({"rows": "stored coupling values (row kernel)",
+                                    "owner": "stored coupling values (owner/gather passes)",
+                                    "subgroup": "factorised: radial band products x angular coefficients, subgroup form",
+                                    "channel": "factorised: radial band products x angular coefficients, per-channel form",
+                                    "angular": "factorised: angular sums first"}
+                                   [forms["apply32"]] if args.precision == 2 else None),
                    "assembly": "overlapped with the previous step's solve" if (args.precision == 2 and
                                                                                args.overlap) else "in step",
-                   "l2": "inputs larger than L2: %.1f GB of coupling values streamed per operator apply" %
-                         (8 * coup / 1e9),
+                   "l2": l2_note(bas, cfg, forms),
                    "parallelism": "replicas x%d (independent instances, no collective)" % world},
         "iters_per_step": float(np.mean(its)), "max_resid": float(np.max(res)),
         "host_loop": {"value": args.steps / (ms_host / 1000.0), "ms_per_step": ms_host / args.steps,
