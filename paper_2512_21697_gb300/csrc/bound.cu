@@ -48,7 +48,7 @@ __global__ void k_pbound(OpView A, const double2* __restrict__ psi, const double
         sx[i] = acc;
     }
     __syncthreads();
-    // four vectors per warp and round, added in ascending order: 63 -> PBNEW us at 144 channels, 302 slots
+    // four vectors per warp and round, added in ascending order: 63 -> 35 us at 144 channels, 302 slots
     // against a block-wide sum per vector
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = PB_T / 32, b1 = bstart[ks + 1];
     double tot = 0;

@@ -741,9 +741,12 @@ static dirac_status alloc_krylov(dirac_op* op, Krylov& K, int prec, double tol)
 // .. 1000, l <= 1 .. 6, all mu and |mu| = 1/2, a call that assembles its time (stored time / factorised
 // time): from q = 40e3 on the residual gains 1.32 (|kappa| <= 10, N = 600, l <= 1) to 2.77 (production,
 // q = 143e3) and the complex64 apply 3.2 to 9; at 15e3 .. 25e3 the residual ranges over 0.90 .. 1.27.  In
-// FP64 the apply alone, of which a step has ten for one assembly, ranges over 0.94 (|kappa| <= 20, N = 250,
-// l <= 6) .. 1.66 above q = 85e3 and is the slower one below (0.59 .. 0.96 at 60e3 .. 84e3).  Few channels
-// per kappa (|mu| = 1/2) leave the lanes idle: q stays below 11e3 there.
+// FP64 the apply alone ranges over 0.84 .. 1.66 above q = 85e3 and is the slower one below (0.59 .. 0.96 at
+// 60e3 .. 84e3); it loses above where the radial pass ends in a nearly empty round of the chip (|kappa| <=
+// 20, N = 250, l <= 6: 1.94 against 1.62 ms; |kappa| <= 24: 2.86 against 2.55).  A step has 4 to 6 applies
+// for one assembly, which the stored form takes 2.3 and 3.5 ms for there: steps of this form are the faster
+// ones at all eight such systems tried (three pulse phases and fields each).  Few channels per kappa (|mu| =
+// 1/2) leave the lanes idle: q stays below 11e3 there.
 static bool ang_pays(const dirac_op* op)
 {
     const int n1 = op->B.n1;   // (the view is not set yet)
