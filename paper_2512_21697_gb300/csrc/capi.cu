@@ -1177,12 +1177,14 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
             hL[(size_t)ks * ns * kb + e] = make_double2(lu.L[e].real(), lu.L[e].imag());
         std::copy(lu.piv.begin(), lu.piv.end(), hP.begin() + (size_t)ks * ns);
     }
-    // in FP64 the warp schedules take U's rows divided by their diagonals (column form)
+    // in FP64 the warp schedules take U's rows divided by their diagonals (column form).  fma(a, b, 0) is the
+    // rounded product: written as a * b, whether it is contracted into the sum depends on the inlining
+    // around it on a host with fused multiply-adds, and with it the last bits of every FP64 solve.
     auto by_diag = [&](int ks, int i, int k) {
-        const size_t e = ((size_t)ks * ns + i) * (wu + 1) + k;
-        const cd u = i - k >= 0 ? cd(hU[e].x, hU[e].y) * cd(hDi[(size_t)ks * ns + i - k].x, hDi[(size_t)ks * ns + i - k].y)
-                                : cd(0);
-        return make_double2(u.real(), u.imag());
+        if (i - k < 0) return make_double2(0, 0);
+        const double2 u = hU[((size_t)ks * ns + i) * (wu + 1) + k], d = hDi[(size_t)ks * ns + i - k];
+        return make_double2(std::fma(u.x, d.x, 0.0) - std::fma(u.y, d.y, 0.0),
+                            std::fma(u.x, d.y, 0.0) + std::fma(u.y, d.x, 0.0));
     };
     std::vector<double2> hUs(hU.size());
     for (int ks = 0; ks < nk2; ks++)
