@@ -332,7 +332,8 @@ dirac_status dirac_op_set_overlap(dirac_op* op, int enable);
  * form (six operations: every accumulator starts from an offset 1.5 * 2^k with 2^(k-2) at least a
  * bound of its sum of |products|, formed each pass from the coupling's static envelopes, the
  * pulse factors and the current vectors; error of order 2^-48 times the offset, so about
- * 1e-13 ||b|| on strong-field random states); mode 0 (the default) takes mode 2 when the solver
+ * 1e-13 ||b|| on strong-field random states and 2e-13 to 1.6e-12 ||b|| on a propagated state, whose
+ * residual is small against the bounds); mode 0 (the default) takes mode 2 when the solver
  * tolerance is at least 1e-11 and mode 1 below.  Both end on the same accurate residual test.
  * DIRAC_E_ARG for other modes. */
 dirac_status dirac_op_set_residual_mode(dirac_op* op, int mode);

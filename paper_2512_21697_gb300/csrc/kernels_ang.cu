@@ -40,9 +40,11 @@
 //   complex64      0.24 + 0.33 ms   subgroup form 1.03 ms, stored owner/gather form 1.56 ms
 //   double-float   0.93 + 1.50 ms   owner + gather passes 3.12 + 0.61 ms
 //   FP64           3.95 + 8.14 ms   row kernel 15.6 ms
-// The FP64 one is bound by the FP64 pipe: 6.4e9 multiply-adds take 10 ms at 0.62e12 a second.  The other
-// two are bound by issue and latency, two blocks of k_rad an SM (its 2 x RSL complex accumulators and
-// window in registers): 6.4e9 multiply-adds of FP32 alone would take 0.17 ms.
+// Counters at 420 channels and 601 slots: the FP64 one holds the FP64 pipe at 97 % in both passes.  The
+// double-float one has the FMA pipe at 46 (k_ang) and 54 % (k_rad) with the offsets, 64 and 71 % as Dot2 sums, and
+// latency for the rest: k_rad's 2 x RSL complex accumulators and window in registers leave two blocks an
+// SM.  The complex64 one is bound by latency (FMA pipe 23 and 29 %): 6.4e9 multiply-adds of FP32 alone
+// would take 0.17 ms at the size above.
 #include <cuda_runtime.h>
 
 #include <algorithm>
