@@ -951,7 +951,7 @@ static dirac_status ang_setup(dirac_op* op)
 
 // Whether a single product (dirac_apply, dirac_apply32, dirac_residual) takes the angular sums first.  Where
 // the steps keep the stored form, the first such product sets the tables up (at 1860 channels, 1001 slots
-// and seven multipoles 1.3 GB beside 21.8, in 15 ms), so that an op which only steps holds none of them.
+// and seven multipoles 1.3 GB beside 21.7, in 15 ms), so that an op which only steps holds none of them.
 // Nothing is allocated while the op's stream is captured, nor where memory is short: the product then takes
 // the stored form.
 static bool call_ang(dirac_op* op)
@@ -1190,11 +1190,10 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     for (int ks = 0; ks < nk2; ks++)
         for (int i = 0; i < ns; i++)
             for (int k = 0; k <= wu; k++) hUs[((size_t)ks * ns + i) * (wu + 1) + k] = by_diag(ks, i, k);
-    double2 *dU, *dL, *dUr, *dDi;
+    double2 *dU, *dL, *dDi;
     int *dP, *dord;
     TRY(upload(op, &dU, hUs));
     TRY(upload(op, &dL, hL));
-    TRY(upload(op, &dUr, hUr));
     TRY(upload(op, &dDi, hDi));
     TRY(upload(op, &dP, hP));
     // the rotated-lane schedule's tables, entry (row, lane): forward the multiplier of the row that the
@@ -1261,7 +1260,7 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     for (size_t gi = 0; gi < P.g.size(); gi++) std::copy(P.g[gi].v.begin(), P.g[gi].v.end(), hM.begin() + gi * be);
     double* dM;
     TRY(upload(op, &dM, hM));
-    TRY(dev_alloc(op, &op->G, (size_t)P.L * 4 * be));
+    if (!dfloat) TRY(dev_alloc(op, &op->G, (size_t)P.L * 4 * be));
     TRY(dev_alloc(op, &op->s, (size_t)P.L * 3));
     TRY(dev_alloc(op, &op->t_eval, 1));
     op->pv.L = P.L;
@@ -1373,7 +1372,7 @@ extern "C" dirac_status dirac_operator_setup(const dirac_basis* basis, const dir
     // Krylov workspaces and reduction partials
     TRY(alloc_krylov(op, op->k64, 0, opts->tol));
     op->k64.S = dS; op->k64.H = dH; op->k64.W = op->W; op->k64.U = dU; op->k64.L = dL;
-    op->k64.Urow = dUr; op->k64.Dinv = dDi;
+    op->k64.Dinv = dDi;
     op->k64.rotF = dRF; op->k64.rotB = dRB;
     if (mixed) {
         if (!dfloat) TRY(dev_alloc(op, &op->W32, wlen));

@@ -21,7 +21,7 @@ struct Krylov {
          *sv = nullptr, *sh = nullptr, *t = nullptr;
     KState* ks = nullptr;
     const void *S = nullptr, *H = nullptr, *W = nullptr, *U = nullptr, *L = nullptr;
-    const void *Urow = nullptr, *Dinv = nullptr;   // lane-per-channel preconditioner data
+    const void *Urow = nullptr, *Dinv = nullptr;   // U by rows (complex64, lane-per-channel schedule); 1 / diagonal
     const void *rotF = nullptr, *rotB = nullptr;   // rotated-lane preconditioner's factor tables
 };
 
